@@ -514,7 +514,11 @@ VG_API int vg_profile_read(vg_grid *grid, double ms[VG_NKERNELS], int64_t timed[
  *                    16 or 32, or 0 for automatic (the default: the fewest
  *                    lanes, at least 8, whose share of the longest ray is
  *                    at most 1.5 times the per-lane buffer of runs of
- *                    visits).  Results do not depend on it.
+ *                    visits).  Results do not depend on it.  Large frames
+ *                    trace without walking (K3 finds each ray's first
+ *                    occupied voxel, K4 looks its rays up per voxel) unless
+ *                    VG_FLAG_STATS counts visits; this knob, K3's CTAs per
+ *                    SM and K4's words then have no effect.
  *  VG_TUNE_INFLATE_TILE
  *                    K2's tile of plane words: VG_TILE_AUTO (the default:
  *                    8 words x 8 rows x 8 slices, 4 slices when the grid has

@@ -15,11 +15,12 @@ namespace {
 
 template <int R, int TXW, int TY, int TZ>
 __global__ void __launch_bounds__(256) k_inflate(const PlaneGeom g, const uint32_t *__restrict__ raw,
-                                                 uint32_t *__restrict__ out, const int r_rt) {
+                                                 uint32_t *__restrict__ out, const int r_rt, const int3 first) {
     extern __shared__ uint32_t sm[];
     pdl_trigger();
     pdl_wait();
-    units::inflate_tile<R, TXW, TY, TZ, units::LoadRO>(g, raw, out, r_rt, blockIdx.x, blockIdx.y, blockIdx.z, sm);
+    units::inflate_tile<R, TXW, TY, TZ, units::LoadRO>(g, raw, out, r_rt, first.x + blockIdx.x, first.y + blockIdx.y,
+                                                       first.z + blockIdx.z, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -53,12 +54,13 @@ __host__ __device__ constexpr int tma_box_words() { return (TXW + 8) * (TY + 2 *
 
 template <int R, int TXW, int TY, int TZ>
 __global__ void __launch_bounds__(256) k_inflate_tma(const __grid_constant__ CUtensorMap tm, const PlaneGeom g,
-                                                     uint32_t *__restrict__ out) {
+                                                     uint32_t *__restrict__ out, const int3 first) {
     constexpr int BW = TXW + 8, HY = TY + 2 * R, HZ = TZ + 2 * R;
     constexpr uint32_t kBytes = (uint32_t)tma_box_words<R, TXW, TY, TZ>() * 4u;
     extern __shared__ __align__(128) uint32_t sm[];   // the box, then the x pass's HZ * HY * TXW words
     __shared__ __align__(8) uint64_t bar;
     pdl_trigger();
+    const int tx = first.x + (int)blockIdx.x, ty = first.y + (int)blockIdx.y, tz = first.z + (int)blockIdx.z;
     const uint32_t b = smem_addr(&bar);
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
@@ -67,7 +69,7 @@ __global__ void __launch_bounds__(256) k_inflate_tma(const __grid_constant__ CUt
     __syncthreads();
     pdl_wait();   // occ_raw is K1's
     if (threadIdx.x == 0) {
-        const int x = (int)blockIdx.x * TXW - 4, y = (int)blockIdx.y * TY - R, z = (int)blockIdx.z * TZ - R;
+        const int x = tx * TXW - 4, y = ty * TY - R, z = tz * TZ - R;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(kBytes) : "memory");
         asm volatile(
             "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
@@ -86,16 +88,24 @@ __global__ void __launch_bounds__(256) k_inflate_tma(const __grid_constant__ CUt
         return;
     }
     // the word w0 - 1 of each staged row is column 3 of the box
-    units::inflate_passes<R, TXW, TY, TZ>(g, out, R, blockIdx.x, blockIdx.y, blockIdx.z, sm, BW, 3,
-                                          sm + BW * HY * HZ);
+    units::inflate_passes<R, TXW, TY, TZ>(g, out, R, tx, ty, tz, sm, BW, 3, sm + BW * HY * HZ);
+}
+
+// The tiles of the frame's box: the first one and how many each way.
+template <int TXW, int TY, int TZ>
+dim3 box_tiles(const WordBox &b, int3 &t0) {
+    t0 = make_int3(b.w0 / TXW, b.y0 / TY, b.z0 / TZ);
+    return dim3((b.w0 + b.nw + TXW - 1) / TXW - t0.x, (b.y0 + b.ny + TY - 1) / TY - t0.y,
+                (b.z0 + b.nz + TZ - 1) / TZ - t0.z);
 }
 
 template <int R, int TXW, int TY, int TZ>
 cudaError_t run(const FrameArgs &a, cudaStream_t s) {
-    dim3 grid((a.g.wx + TXW - 1) / TXW, (a.g.ny + TY - 1) / TY, (a.g.nz + TZ - 1) / TZ);
+    int3 t0;
+    const dim3 grid = box_tiles<TXW, TY, TZ>(a.box, t0);
     const size_t bytes = sizeof(uint32_t) * units::inflate_smem_words<R, TXW, TY, TZ>(a.r);
     return launch_pdl(k_inflate<R, TXW, TY, TZ>, grid, 256, bytes, s, a.g, (const uint32_t *)a.pl.occ_raw,
-                      a.pl.occ_inf, a.r);
+                      a.pl.occ_inf, a.r, t0);
 }
 
 // The driver's tensor-map encoder, looked up once through the runtime (the
@@ -169,9 +179,10 @@ template <int R, int TXW, int TY, int TZ>
 cudaError_t run_tma(const FrameArgs &a, cudaStream_t s) {
     CUtensorMap m;
     if (!plane_map(a.pl.occ_raw, a.g, TXW + 8, TY + 2 * R, TZ + 2 * R, m)) return run<R, TXW, TY, TZ>(a, s);
-    dim3 grid((a.g.wx + TXW - 1) / TXW, (a.g.ny + TY - 1) / TY, (a.g.nz + TZ - 1) / TZ);
+    int3 t0;
+    const dim3 grid = box_tiles<TXW, TY, TZ>(a.box, t0);
     const size_t bytes = sizeof(uint32_t) * (tma_box_words<R, TXW, TY, TZ>() + (TZ + 2 * R) * (TY + 2 * R) * TXW);
-    return launch_pdl(k_inflate_tma<R, TXW, TY, TZ>, grid, 256, bytes, s, m, a.g, a.pl.occ_inf);
+    return launch_pdl(k_inflate_tma<R, TXW, TY, TZ>, grid, 256, bytes, s, m, a.g, a.pl.occ_inf, t0);
 }
 
 template <int TXW, int TZ>
@@ -223,8 +234,9 @@ cudaError_t launch_inflate(const FrameArgs &a, cudaStream_t s, const Sched &sc) 
     const bool wide_ok = a.g.wx % 8 == 0;
     int tile = sc.inflate_tile;
     if (tile == kTileAuto) {
-        const int txw = wide_ok ? 8 : 4;
-        const int64_t tiles8 = (int64_t)((a.g.wx + txw - 1) / txw) * ((a.g.ny + 7) / 8) * ((a.g.nz + 7) / 8);
+        int3 t0;
+        const dim3 t = wide_ok ? box_tiles<8, 8, 8>(a.box, t0) : box_tiles<4, 8, 8>(a.box, t0);
+        const int64_t tiles8 = (int64_t)t.x * t.y * t.z;
         const int64_t sms = sms_of_current_device();
         const bool short_tiles = tiles8 >= sms && tiles8 < 4 * sms;
         tile = wide_ok ? (short_tiles ? kTile8x8x4 : kTile8x8x8) : (short_tiles ? kTile4x8x4 : kTile4x8x8);

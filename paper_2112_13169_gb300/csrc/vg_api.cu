@@ -32,7 +32,7 @@ struct vg_grid {
     int device;
     uint8_t *base;        // the one device allocation
     uint8_t *loc;         // ring-addressed by ring (vg::Ring)
-    uint8_t *loc_alt;     // staging for reads into memory the device cannot store to
+    uint8_t *loc_alt;     // staging for reads into memory the device cannot store to; a gathered frame's tables
     // A re-centre by d (o' = o + d) moves the ring by d at once; the voxels
     // it brings in still hold stale bytes until the next merge sets them to
     // unknown (a read treats them as unknown meanwhile): pend = d while that
@@ -223,11 +223,19 @@ FrameArgs frame_args(vg_grid *G, const vg::Pose32 &T) {
     return a;
 }
 
+// Takes the gathered form where the frame allows it and it pays, its tables
+// in loc_alt (which a read only stages through, in stream order).  Counting
+// visits and the literal readings need the walk itself.
+void gather_form(const vg_grid *G, FrameArgs &a) {
+    if (G->p.flags == 0 && vg::host::gather_pays(a)) vg::host::gather_setup(a, G->loc_alt, (size_t)G->g.nvox + 16);
+}
+
 // FrameArgs of a depth frame: the pinhole intrinsics from the field of view.
 FrameArgs depth_frame_args(vg_grid *G, const vg::Pose32 &T, const void *depth, int32_t width, int32_t height,
                            int32_t dtype, float depth_scale) {
     FrameArgs a = frame_args(G, T);
     vg::host::set_depth_frame(a, &G->p, depth, width, height, dtype, depth_scale);
+    gather_form(G, a);
     return a;
 }
 
@@ -289,7 +297,6 @@ cudaError_t apply_pending(vg_grid *G, cudaStream_t s) {
 }
 
 // K2..K4 after K1 has filled occ_raw.
-
 cudaError_t finish_frame(vg_grid *G, FrameArgs &a, cudaStream_t s) {
     cudaError_t e;
     if (a.r > 0) {
@@ -297,6 +304,17 @@ cudaError_t finish_frame(vg_grid *G, FrameArgs &a, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     } else {
         a.pl.occ_inf = a.pl.occ_raw;   // no inflation: the raw plane is the inflated one
+    }
+    if (a.ga.on) {
+        // (two launches under one kernel id: the hits, and what K4 looks up of them)
+        e = launch(G, VG_K_RAYTRACE, s, [&] { return vg::launch_rayhit(a, s); });
+        if (e != cudaSuccess) return e;
+        ++G->launches[VG_K_RAYTRACE];
+        a.ring = ring_of(G);
+        e = launch(G, VG_K_MERGE, s, [&] { return vg::launch_gather(a, s); });
+        if (e != cudaSuccess) return e;
+        G->pend_on = false;
+        return cudaSuccess;
     }
     // the plane the rays test: the inflated one (Alg. 1's order), or a
     // literal reading's
@@ -644,6 +662,7 @@ int vg_integrate_points(vg_grid *G, const float *xyz, int32_t mem, int64_t n, co
     FrameArgs a = frame_args(G, T);
     a.xyz = static_cast<const float *>(dptr);
     a.npts = n;
+    gather_form(G, a);
     cudaError_t e = launch(G, VG_K_VOXELIZE, s, [&] { return vg::launch_voxelize_points(a, s, G->sched); });
     if (e == cudaSuccess) e = finish_frame(G, a, s);
     if (e != cudaSuccess) return status_of(e);
@@ -905,6 +924,7 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
         vg::BatchItem &it = items[i];
         std::memset(&it, 0, sizeof(it));
         it.a = depth_frame_args(G, T, f.depth, f.width, f.height, f.dtype, f.depth_scale);
+        it.a.ga.on = 0;
         if (G->p.vox_inf == 0) it.a.pl.occ_inf = it.a.pl.occ_raw;
         it.a.occ_test = it.a.pl.occ_inf;
         it.dtype = f.dtype;

@@ -15,6 +15,7 @@
 #include "vg.h"
 #include "vg_internal.cuh"
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -126,8 +127,11 @@ inline FrameArgs frame_args(const vg_params *p, const PlaneGeom &g, const Pose32
     a.depth_max = p->depth;
     bundle_of(p, a.vd, a.hw, a.hh);
     a.r = p->vox_inf;
+    a.box = {0, g.wx, 0, g.ny, 0, g.nz};
     return a;
 }
+
+inline void depth_box(FrameArgs &a, const vg_params *p);
 
 // Adds a depth frame's input and pinhole intrinsics to a.
 inline void set_depth_frame(FrameArgs &a, const vg_params *p, const void *depth, int32_t width, int32_t height,
@@ -140,6 +144,111 @@ inline void set_depth_frame(FrameArgs &a, const vg_params *p, const void *depth,
     a.fy = (float)(((double)height / 2.0) / tan(half_fov(p->fov_y_deg)));
     a.cx = (float)(((double)width - 1.0) / 2.0);
     a.cy = (float)(((double)height - 1.0) / 2.0);
+    depth_box(a, p);
+}
+
+// Narrows a depth frame's box to what its pixels (inflated by vox_inf) and
+// rays can reach: the pyramid of both from the camera, with two voxels to
+// spare for rounding.  Poses whose rotation block is no rotation keep their
+// linear map, so the corners bound it all the same.
+inline void depth_box(FrameArgs &a, const vg_params *p) {
+    const double d = std::max((double)a.vd, (double)p->depth / (double)p->vox_size);
+    const double kx = std::max(tan(half_fov(p->fov_x_deg)), a.vd > 0 ? (double)a.hw / a.vd : 0.0) * d;
+    const double ky = std::max(tan(half_fov(p->fov_y_deg)), a.vd > 0 ? (double)a.hh / a.vd : 0.0) * d;
+    int32_t lo[3], hi[3];
+    const int32_t n[3] = {a.g.nx, a.g.ny, a.g.nz};
+    for (int k = 0; k < 3; ++k) {
+        const double s = (double)a.T.t[k] / (double)a.vs;
+        const double fwd = (double)a.T.R[k * 3 + 2] * d;
+        const double side = std::fabs((double)a.T.R[k * 3]) * kx + std::fabs((double)a.T.R[k * 3 + 1]) * ky;
+        const double spare = a.r + 2.0 + 1e-6 * (std::fabs(s) + std::fabs(fwd) + side);
+        lo[k] = (int32_t)std::min(std::max(floor(s + std::min(0.0, fwd - side) - spare), 0.0), (double)n[k]);
+        hi[k] = (int32_t)std::min(std::max(ceil(s + std::max(0.0, fwd + side) + spare), 0.0), (double)n[k]);
+        if (hi[k] < lo[k]) hi[k] = lo[k];
+    }
+    if (lo[0] == hi[0] || lo[1] == hi[1] || lo[2] == hi[2]) {   // nothing of the grid: one word, for the launches
+        a.box = {0, 1, 0, 1, 0, 1};
+        return;
+    }
+    a.box = {lo[0] / 32, (hi[0] + 31) / 32 - lo[0] / 32, lo[1], hi[1] - lo[1], lo[2], hi[2] - lo[2]};
+}
+
+// Whether the gathered form of a frame (vg_gather.cuh) is the faster one:
+// its voxels, the smaller of the bundle's pyramid and half its box, number
+// kGatherVoxels or more.  Its kernels take about as long as the scattered
+// ones of 10,700 rays of 71 voxels (252 k by this count; 640x480 frames of a
+// 10 x 10 x 5 m grid: 36.1 against 36.0 us a frame with its read); below, the
+// fixed cost of the lists and of one launch more is not made up (8,295 rays
+// of 43 voxels: 28 against 22 us), above it is (21,201 of 100: 41.4 against
+// 45.3; 33,221 of 125: 56 against 70; 132,525 of 250: 163 against 350).
+constexpr double kGatherVoxels = 250e3;
+inline bool gather_pays(const FrameArgs &a) {
+    const double rays = (2.0 * a.hw + 1.0) * (2.0 * a.hh + 1.0);
+    const double box = 32.0 * a.box.nw * a.box.ny * a.box.nz;
+    return std::min(rays * a.vd / 3.0, box / 2.0) >= kGatherVoxels;
+}
+
+// Sets up the gathered form of a frame (vg_gather.cuh) in `bytes` bytes of
+// device memory at base (256-byte aligned), or leaves it off: a.T, a.vs, the
+// bundle and the geometry are set.  The form needs a rotation (within 1e-3:
+// a voxel's inscribed sphere stays one), a bundle of at most 105 degrees (a wider one
+// crosses voxels outside the near words at depths where windows are huge) and
+// a camera, grid and range within 4096 voxels, so that float coordinates in
+// camera axes (off by at most about 4096 * 2^-22 * 10) stay well inside
+// kGatherMargin, and room for its tables: 20 bytes a ray, 4 a tile of 64 and the
+// near words.
+// Other frames take the scattered form.
+inline void gather_setup(FrameArgs &a, uint8_t *base, size_t bytes) {
+    Gather &g = a.ga;
+    g.on = 0;
+    if (a.vd < 1 || a.vd > 4096 || a.hw > 1.3 * a.vd || a.hh > 1.3 * a.vd) return;
+    const int32_t n[3] = {a.g.nx, a.g.ny, a.g.nz};
+    double R[9], M[9];
+    for (int k = 0; k < 9; ++k) R[k] = a.T.R[k];
+    for (int i = 0; i < 3; ++i) {
+        if (n[i] > 4096 || !(std::fabs(a.T.t[i] / a.vs) <= 4096.0f)) return;
+        for (int j = 0; j < 3; ++j) {
+            const double d = R[i] * R[j] + R[3 + i] * R[3 + j] + R[6 + i] * R[6 + j];
+            if (!(std::fabs(d - (i == j ? 1.0 : 0.0)) <= 1e-3)) return;
+        }
+    }
+    for (int i = 0; i < 3; ++i)
+        for (int j = 0; j < 3; ++j) {   // adjugate
+            const int i1 = (i + 1) % 3, i2 = (i + 2) % 3, j1 = (j + 1) % 3, j2 = (j + 2) % 3;
+            M[j * 3 + i] = R[i1 * 3 + j1] * R[i2 * 3 + j2] - R[i1 * 3 + j2] * R[i2 * 3 + j1];
+        }
+    const double det = R[0] * M[0] + R[1] * M[3] + R[2] * M[6];
+    for (int k = 0; k < 9; ++k) M[k] /= det;
+
+    const int64_t rays = (2 * (int64_t)a.hw + 1) * (2 * (int64_t)a.hh + 1);
+    const int64_t tiles = (int64_t)((2 * a.hw + 8) >> 3) * ((2 * a.hh + 8) >> 3);
+    if (!base || rays * 20 + tiles * 4 + 2 * kNearWords * 4 > (int64_t)bytes || rays >= (int64_t(1) << 30)) return;
+    g.rays = (int32_t)rays;
+    g.inv = reinterpret_cast<float4 *>(base);
+    g.hit = reinterpret_cast<uint32_t *>(g.inv + rays);
+    g.tile = g.hit + rays;
+    g.near_fr = g.tile + tiles;
+    g.near_tr = g.near_fr + kNearWords;
+
+    const double ka = (double)a.hw / a.vd, kb = (double)a.hh / a.vd;
+    g.ka = (float)ka;
+    g.kb = (float)kb;
+    for (int side = 0; side < 4; ++side) {
+        const double *m = M + 3 * (side >> 1), k = (side >> 1 ? kb : ka) * (side & 1 ? -1.0 : 1.0);
+        const double c[3] = {std::fabs(m[0] - k * M[6]), std::fabs(m[1] - k * M[7]), std::fabs(m[2] - k * M[8])};
+        const double margin = kGatherMargin * (1.0 + std::fabs(k));
+        g.ew[side] = (float)(16.0 * c[0] + 0.5 * c[1] + 0.5 * c[2] + margin);
+        g.ep[side] = (float)(4.0 * c[0] + 2.0 * c[1] + 0.5 * c[2] + margin);
+        g.ev[side] = (float)(0.5 * (c[0] + c[1] + c[2]) + margin);
+    }
+    for (int k = 0; k < 9; ++k) g.M[k] = (float)M[k];
+    g.zp = (float)(4.0 * std::fabs(M[6]) + 2.0 * std::fabs(M[7]) + 0.5 * std::fabs(M[8]));
+    g.zw = (float)(16.0 * std::fabs(M[6]) + 0.5 * std::fabs(M[7]) + 0.5 * std::fabs(M[8]));
+    g.zv = (float)(0.5 * (std::fabs(M[6]) + std::fabs(M[7]) + std::fabs(M[8])));
+    // |a - fa| <= vd (reach + margin) / (c2 - zv - margin) + margin, as in window_of
+    const double reach = std::max(std::max(g.ev[0], g.ev[1]), std::max(g.ev[2], g.ev[3]));
+    g.zr = (float)(a.vd * reach / (kLateReach - 0.5 - 2.0 * kGatherMargin) + g.zv + 2.0 * kGatherMargin);
+    g.on = 1;
 }
 
 }  // namespace host

@@ -3,7 +3,8 @@
 // Device data layout of one grid (one cudaMalloc, carved in this order):
 //   loc      Nx*Ny*Nz bytes, the paper's index order idx = x + y*Nx + z*Nx*Ny,
 //            followed by at least 16 bytes of slack
-//   loc_alt  the same size; target of the out-of-place shift (ping-pong)
+//   loc_alt  the same size; staging of reads, and between K1 and K4 of a
+//            gathered frame its tables (Gather)
 //   occ_raw, occ_inf, fr, tr
 //            bit planes of the measurement grid.  Bit b of word
 //            (z*Ny + y)*WX + w is voxel x = 32*w + b of row (y, z), i.e.
@@ -91,6 +92,36 @@ struct Ring {
     int32_t elo[3], ehi[3];
 };
 
+// The part of a grid a frame can mark or occupy: words [w0, w0 + nw) of rows
+// [y0, y0 + ny) of slices [z0, z0 + nz).  Everything outside is unoccupied.
+struct WordBox {
+    int32_t w0, nw, y0, ny, z0, nz;
+};
+
+// The gathered form of K3 and K4 (vg_gather.cuh): the inverse of the pose's
+// rotation, the widths of a word's and a voxel's projection that its culling
+// compares with, and where its per-frame tables live (in the grid's loc_alt,
+// which holds nothing between calls).
+constexpr float kGatherMargin = 0.03f;   // voxels: bounds the rounding of the bundle coordinates (gather_setup)
+constexpr int kNearReach = 7;            // voxels around the camera's that the rays mark themselves
+constexpr int kLateReach = 3;            // rays around each one whose latest hit is tabled
+constexpr int kNearWords = (2 * kNearReach + 1) * (2 * kNearReach + 1);
+struct Gather {
+    int32_t on;         // 0: the frame takes the scattered form (vg_rt.cuh)
+    int32_t rays;       // rays of the bundle
+    float M[9];         // inverse of T.R
+    float ka, kb;       // slopes of the bundle's sides: hw / vd, hh / vd
+    // reach of a word (ew), a patch of 8 x 4 voxels (ep) or a voxel (ev)
+    // across the sides +a, -a, +b, -b, and along the optical axis
+    float ew[4], ep[4], ev[4];
+    float zw, zp, zv;
+    float zr;           // depth from which a voxel's window lies within kLateReach - 1/2 rays of its centre
+    float4 *inv;        // per ray: 1/D of the walk, 0 on an inactive axis; the latest hit around it
+    uint32_t *hit;      // per ray: its hit key
+    uint32_t *tile;     // per tile of 8 x 8 rays: the latest hit key
+    uint32_t *near_fr, *near_tr;   // marks of the voxels around the camera, one word per row
+};
+
 struct FrameArgs {
     PlaneGeom g;
     Pose32 T;
@@ -109,12 +140,14 @@ struct FrameArgs {
     int32_t r;         // vox_inf
     Planes pl;
     uint8_t *loc;
+    WordBox box;                // K2's tiles and the gathered form's words
     Ring ring;                  // loc's ring addressing, with the voxels a re-centre brought in
     unsigned long long *stats;  // NULL unless VG_FLAG_STATS
     uint32_t *rt_next;          // K3's counter of handed-out bundles, zeroed by K1; NULL: static only
     // literal readings (comparison flags; 0 for the default reading)
     const uint32_t *occ_test;   // the plane K3's rays test; NULL: pl.occ_inf
     int32_t lit;                // kLit* bits
+    Gather ga;
 };
 
 constexpr int32_t kLitSkipStart = 1;    // rays do not visit their start voxel
@@ -133,6 +166,8 @@ struct BatchItem {
     int32_t tz;         // inflate tile height in slices: 4 or 8
     int32_t mwpu;       // plane words per phase-4 unit: 256 or 512
     int32_t buffered;   // packed runs fit (plane words < kRunWords)
+    int32_t near_units; // gathered form: phase-3 units that mark the voxels around the camera
+    int32_t pad;
     int64_t woff3;      // phase 3: weight of the units before this frame's
     int64_t w3;         // phase 3: weight of each of this frame's units
 };
@@ -187,6 +222,9 @@ cudaError_t configure_inflate();   // once per device, before the first launch_i
 // device waits of K2 that ran out on the current device since the library was loaded
 cudaError_t wait_timeouts(unsigned *out);
 cudaError_t launch_inflate(const FrameArgs &a, cudaStream_t s, const Sched &sc = Sched());
+// the gathered form's K3 and K4 (a.ga.on; k_gather.cu)
+cudaError_t launch_rayhit(const FrameArgs &a, cudaStream_t s);
+cudaError_t launch_gather(const FrameArgs &a, cudaStream_t s);
 cudaError_t configure_raytrace(int dev);   // once per device, before the first launch_raytrace
 int auto_lanes_per_ray(int32_t vd, int32_t hw, int32_t hh);
 cudaError_t launch_raytrace(const FrameArgs &a, int lanes_per_ray, cudaStream_t s, const Sched &sc = Sched());

@@ -107,11 +107,22 @@ extern "C" VG_API int vg_integrate_depth_noalloc(const vg_params *params, const 
     a.loc = dloc;
     a.stats = nullptr;
 
+    // the gathered form's tables take the place of the fr and tr planes,
+    // which it has none of
+    if (vg::host::gather_pays(a))
+        vg::host::gather_setup(a, reinterpret_cast<uint8_t *>(scratch + 2 * g.words),
+                               (size_t)(4 * kPlaneWords - 2 * g.words) * sizeof(uint32_t));
+
     // the planes must start empty; the array holds whatever the last call left
-    e = cudaMemsetAsync(scratch, 0, (size_t)(4 * g.words) * sizeof(uint32_t), s);
+    e = cudaMemsetAsync(scratch, 0, (size_t)((a.ga.on ? 2 : 4) * g.words) * sizeof(uint32_t), s);
     if (e == cudaSuccess) e = vg::launch_voxelize_depth(a, dtype, s);
     if (e == cudaSuccess && a.r > 0) e = vg::launch_inflate(a, s);
     if (e == cudaSuccess && a.r == 0) a.pl.occ_inf = a.pl.occ_raw;
+    if (a.ga.on) {
+        if (e == cudaSuccess) e = vg::launch_rayhit(a, s);
+        if (e == cudaSuccess) e = vg::launch_gather(a, s);
+        return vg::host::status_of(e);
+    }
     if (e == cudaSuccess)
         e = vg::launch_raytrace(a, vg::auto_lanes_per_ray(a.vd, a.hw, a.hh), s);
     if (e == cudaSuccess) e = vg::launch_merge(a, s);
