@@ -112,9 +112,10 @@ struct Layout {
 Layout layout_of(const PlaneGeom &g, uint32_t flags) {
     Layout L;
     size_t off = 0;
-    // 16 bytes of slack after each loc buffer: K5's vector path may read up
-    // to 4 bytes past the last voxel (and discards them)
+    // K5 reads (and discards) up to 15 bytes before loc, which the stats
+    // leave room for, and a few past it, for which 16 bytes are left
     const size_t locb = align256((size_t)g.nvox + 16), planeb = align256((size_t)g.words * 4);
+    L.stats = off; off += 256;
     L.loc = off; off += locb;
     L.loc_alt = off; off += locb;
     L.occ_raw = off; off += planeb;
@@ -123,7 +124,6 @@ Layout layout_of(const PlaneGeom &g, uint32_t flags) {
     L.tr = off; off += planeb;
     L.loc_occ = off;   // only for the literal loc_grid reading
     if (flags & VG_FLAG_LIT_LOC_OCCUPANCY) off += planeb;
-    L.stats = off; off += 256;
     L.total = off;
     return L;
 }

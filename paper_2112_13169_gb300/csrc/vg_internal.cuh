@@ -1,6 +1,7 @@
 // vg_internal.cuh -- types shared by the kernels and the host library.
 //
 // Device data layout of one grid (one cudaMalloc, carved in this order):
+//   stats    256 bytes: three u64 counters (VG_FLAG_STATS), K3's counter
 //   loc      Nx*Ny*Nz bytes, the paper's index order idx = x + y*Nx + z*Nx*Ny,
 //            followed by at least 16 bytes of slack
 //   loc_alt  the same size; staging of reads, and between K1 and K4 of a
@@ -11,7 +12,6 @@
 //            plane bit (z*Ny + y)*32*WX + x.  WX is ceil(Nx/32) rounded up
 //            to a power of two, at least 4 words, so every row starts on a
 //            16-byte boundary.  Bits with x >= Nx stay 0.
-//   stats    three u64 counters (VG_FLAG_STATS)
 // The planes are all-zero between frames: K4 clears every word it reads.
 #pragma once
 

@@ -123,3 +123,31 @@ def test_scattered_form_at_gathered_sizes(vg, lanes):
         P.o.shift(f.robot_pos)
     assert P.g.stats()["ray_visits"] > 0
     P.g.close()
+
+
+@pytest.mark.parametrize("n", [(1, 5, 3), (7, 9, 4), (15, 4, 5), (16, 4, 4), (17, 6, 3), (33, 5, 5), (64, 3, 7)])
+def test_reads_through_the_ring(vg, n):
+    # rows shorter than a chunk, of a chunk, and ragged; every wrap position,
+    # read with and without voxels that a re-centre brought in
+    g = vg.Grid(n, 1.0, 60.0, 50.0, 3.0, 0, (0.0, 0.0, 0.0))
+    o = OracleGrid(OracleParams(n, 1.0, 60.0, 50.0, 3.0, 0), (0.0, 0.0, 0.0))
+    rng = np.random.default_rng(n[0])
+    src = rng.integers(0, 4, (n[2], n[1], n[0])).astype(np.uint8)
+    out = torch.full((g.nvox + 32,), 9, dtype=torch.uint8, device="cuda")
+    g.write(src, g.origin)
+    o.loc[:] = src
+    pos = np.zeros(3)
+    for k in range(20):
+        pos = pos + rng.integers(-2, 3, 3)
+        g.shift(pos)
+        o.shift(pos)
+        origin = g.read(out)
+        torch.cuda.synchronize()
+        got = out.cpu().numpy()
+        assert list(origin) == list(o.o)
+        assert_same(got[:g.nvox], o.loc, "read %d of %s" % (k, n))
+        assert (got[g.nvox:] == 9).all()   # nothing past the grid
+        if k % 5 == 4:
+            o.loc[:] = src
+            g.write(src, g.origin)
+    g.close()
