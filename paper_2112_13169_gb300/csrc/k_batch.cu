@@ -2,13 +2,19 @@
 //
 // One cooperative launch of k_batch runs, for every frame of a batch (each
 // with its own grid, resolution, voxel size and radius), the whole path:
-//   phase 1  K1 voxelize           units of 1024 pixels
+//   phase 1  K1 voxelize           units of 1024 pixels; 256 rays of the table
 //   phase 2  K2 inflate            8 (or 4) words x 8 rows x 8 (or 4)
-//                                  slices (radius 1..3)
-//   phase 3  K3 ray trace          groups of at most 256 / LPR rays (a
+//                                  slices (radius 1..3) of the frame's box
+//   phase 3  K3 gathered           256 rays around the camera; 256 words
+//            K3 scattered          groups of at most 256 / LPR rays (a
 //                                  frame's rays spread over its units)
-//   phase 4  K4 merge              512 plane words (256 if tuned)
-// with a grid-wide barrier between phases.  A frame's re-centre (K5) is not
+//   phase 3b K3 gathered           32 x 8 rays (their latest hits)
+//   phase 4  K4 gathered           128 plane words of the box; 256 of slabs
+//            K4 merge              512 plane words (256 if tuned)
+// with a grid-wide barrier between phases (3b only if a frame is gathered).
+// Every frame that the gathered form can take (vg_gather.cuh) takes it here:
+// many frames fill the device, so its fewer instructions count and the
+// latency of its phases does not (the one-frame launch has a rule on sizes).  A frame's re-centre (K5) is not
 // a phase: it moves its grid's ring, and that grid's next merge sets the
 // voxels it brought in to unknown (Ring).
 // Units of every frame are laid end to end per phase (BatchItem::off).  A
@@ -22,6 +28,7 @@
 // tuned): if the other CTAs do not all arrive in time, the waiting CTA sets
 // BatchCtl::error and every CTA leaves the kernel, so the host sees
 // VG_ETIMEOUT instead of a hung GPU.  The launch is cooperative, so all CTAs are resident together.
+#include "vg_gather.cuh"
 #include "vg_rt.cuh"
 #include "vg_sync.cuh"
 
@@ -35,7 +42,12 @@ using namespace rt;
 constexpr int kInflateUnroll = 2;
 constexpr int kDynWords = kRtBuf * kThreads;   // also covers an inflate tile of radius <= 3
 static_assert(units::inflate_smem_words<3, 8, 8, 8>(3) <= (size_t)kDynWords, "inflate tile fits");
+constexpr int kGatherWords = kBatchGatherWords;
+static_assert(sizeof(gather::GatherSmem<kGatherWords>) <= kDynWords * 4, "gathered words fit");
+static_assert(sizeof(gather::SkinSmem) <= kDynWords * 4 && sizeof(gather::LateSmem) <= kDynWords * 4 &&
+              3 * kNearWords <= kDynWords, "gathered K3 fits");
 static_assert(sizeof(FrameArgs) % 4 == 0, "frame arguments copy as words");
+static_assert(sizeof(BatchItem) <= 1024, "the served form's bound on a launch table");
 
 __device__ __forceinline__ int find_item(const BatchItem *items, int n, int phase, int64_t u) {
     int lo = 0, hi = n - 1;
@@ -137,7 +149,12 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
                 __syncthreads();
                 cur = i;
             }
-            const int64_t t = (u - __ldg(&items[i].off[0])) * kThreads + threadIdx.x;
+            const int64_t local = u - __ldg(&items[i].off[0]), pix = __ldg(&items[i].pix_units);
+            const int64_t t = local * kThreads + threadIdx.x;
+            if (local >= pix) {
+                gather::table_thread(s_a, t - pix * kThreads);
+                continue;
+            }
             switch (s_kind) {
             case 0: units::voxelize_depth_thread<0, false>(s_a, t); break;
             case 1: units::voxelize_depth_thread<0, true>(s_a, t); break;
@@ -159,9 +176,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
             // a frame has fewer than 2^27 plane words, so fewer tiles
             const uint32_t local = (uint32_t)(u - it.off[1]), t0 = (uint32_t)it.tiles[0];
             const uint32_t t01 = local / t0;
-            const int tx = (int)(local - t01 * t0);
-            const int ty = (int)(t01 % (uint32_t)it.tiles[1]);
-            const int tz = (int)(t01 / (uint32_t)it.tiles[1]);
+            const int tx = it.tile0[0] + (int)(local - t01 * t0);
+            const int ty = it.tile0[1] + (int)(t01 % (uint32_t)it.tiles[1]);
+            const int tz = it.tile0[2] + (int)(t01 / (uint32_t)it.tiles[1]);
             switch (it.txw * 10 + it.tz) {
             case 88: inflate_unit<8, 8>(it, tx, ty, tz, dyn); break;
             case 84: inflate_unit<8, 4>(it, tx, ty, tz, dyn); break;
@@ -172,10 +189,38 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
     }
     if (!grid_sync(ctl, nb)) return;
 
-    // ---- phase 3: ray trace -----------------------------------------------
+    // ---- phase 3, gathered: around the camera, and the skin ---------------
+    // units in turn over the CTAs: their cost differs between and within
+    // frames.  (Here and in the phases after it frame i's arguments are
+    // staged for every unit: a CTA's units lie far apart.)
+    auto stage = [&](int i) {
+        __syncthreads();   // the previous copy is no longer read
+        stage_args(items[i].a, s_a);
+        __syncthreads();
+    };
+    {
+        float S[3];
+        int32_t v0[3];
+        int i = 0;
+        for (int64_t u = blockIdx.x; u < ctl->total[4]; u += nb) {
+            i = u == blockIdx.x ? find_item(items, n, 4, u) : next_item(items, n, 4, u, i);
+            stage(i);
+            gather::frame_start(s_a, S, v0);
+            const int32_t local = (int32_t)(u - __ldg(&items[i].off[4])), near = __ldg(&items[i].near_units);
+            if (local < near)
+                gather::near_unit<units::LoadPlain>(s_a, S, v0, local, dyn);
+            else
+                gather::skin_unit<units::LoadPlain>(s_a, S, v0, local - near, __ldg(&items[i].skin_units),
+                                                    *reinterpret_cast<gather::SkinSmem *>(dyn));
+        }
+        __syncthreads();
+    }
+
+    // ---- phase 3, scattered: ray trace -------------------------------------
     // a contiguous run of units per CTA, so the camera box is staged again
     // only when the run crosses into another frame; the runs split the
     // units' total weight evenly (weights of 1: their number)
+    if (ctl->total[2])
     {
         const int64_t lo = weighted_unit(items, n, ctl->total[2], run_begin(ctl->wtotal3, blockIdx.x, nb));
         const int64_t hi = weighted_unit(items, n, ctl->total[2], run_begin(ctl->wtotal3, blockIdx.x + 1, nb));
@@ -215,18 +260,44 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
     }
     if (!grid_sync(ctl, nb)) return;
 
+    // ---- phase 3b: the latest hits of the gathered frames' rays -----------
+    if (ctl->total[5]) {
+        int i = 0;
+        for (int64_t u = blockIdx.x; u < ctl->total[5]; u += nb) {
+            i = u == blockIdx.x ? find_item(items, n, 5, u) : next_item(items, n, 5, u, i);
+            stage(i);
+            gather::late_unit<units::LoadPlain>(s_a, (int32_t)(u - __ldg(&items[i].off[5])),
+                                                *reinterpret_cast<gather::LateSmem *>(dyn));
+        }
+        if (!grid_sync(ctl, nb)) return;
+    }
+
     // ---- phase 4: merge ---------------------------------------------------
     {
         // units in turn over the CTAs: their cost differs between frames,
         // and interleaving keeps the CTAs' shares even
+        float S[3];
+        int32_t v0[3];
         int i = find_item(items, n, 3, blockIdx.x);
         for (int64_t u = blockIdx.x; u < ctl->total[3]; u += nb) {
             i = next_item(items, n, 3, u, i);
             const BatchItem &it = items[i];
+            const int64_t local = u - __ldg(&it.off[3]);
+            if (__ldg(&it.a.ga.on)) {
+                stage(i);
+                const int32_t box = __ldg(&it.box_units);
+                if (local < box) {
+                    gather::frame_start(s_a, S, v0);
+                    gather::gather_unit<kGatherWords, units::LoadPlain>(
+                        s_a, S, v0, (uint32_t)local, box, *reinterpret_cast<gather::GatherSmem<kGatherWords> *>(dyn));
+                } else {
+                    gather::slab_word(s_a, (local - box) * kThreads + threadIdx.x);
+                }
+                continue;
+            }
             // the unit's mwpu plane words, one or two per thread
             for (int k = 0; k < it.mwpu; k += kThreads)
-                units::merge_word<units::LoadL2>(it.a.g, it.a.pl, it.a.loc, it.a.ring,
-                                                 (u - it.off[3]) * it.mwpu + k + threadIdx.x);
+                units::merge_word<units::LoadL2>(it.a.g, it.a.pl, it.a.loc, it.a.ring, local * it.mwpu + k + threadIdx.x);
         }
     }
 }

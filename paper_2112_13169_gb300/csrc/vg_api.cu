@@ -7,6 +7,7 @@
 // helpers of vg_host.h).  Everything else runs in the kernels K1..K5,
 // enqueued on the caller's stream without host sync.
 #include "vg.h"
+#include "vg_gather.cuh"
 #include "vg_host.h"
 #include "vg_internal.cuh"
 
@@ -235,7 +236,6 @@ FrameArgs depth_frame_args(vg_grid *G, const vg::Pose32 &T, const void *depth, i
                            int32_t dtype, float depth_scale) {
     FrameArgs a = frame_args(G, T);
     vg::host::set_depth_frame(a, &G->p, depth, width, height, dtype, depth_scale);
-    gather_form(G, a);
     return a;
 }
 
@@ -638,6 +638,7 @@ int vg_integrate_depth(vg_grid *G, const void *depth, int32_t mem, int32_t width
         if (rc != VG_OK) return rc;
     }
     FrameArgs a = depth_frame_args(G, T, dptr, width, height, dtype, depth_scale);
+    gather_form(G, a);
     cudaError_t e = launch(G, VG_K_VOXELIZE, s, [&] { return vg::launch_voxelize_depth(a, dtype, s, G->sched); });
     if (e == cudaSuccess) e = finish_frame(G, a, s);
     if (e != cudaSuccess) return status_of(e);
@@ -915,7 +916,7 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
     }
     vg::BatchCtl *ctl = reinterpret_cast<vg::BatchCtl *>(B->host);
     vg::BatchItem *items = reinterpret_cast<vg::BatchItem *>(B->host + sizeof(vg::BatchCtl));
-    int64_t total[4] = {0, 0, 0, 0};
+    int64_t total[6] = {0, 0, 0, 0, 0, 0};
     for (int32_t i = 0; i < n; ++i) {
         const vg_frame &f = frames[i];
         vg_grid *G = f.grid;
@@ -924,7 +925,11 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
         vg::BatchItem &it = items[i];
         std::memset(&it, 0, sizeof(it));
         it.a = depth_frame_args(G, T, f.depth, f.width, f.height, f.dtype, f.depth_scale);
-        it.a.ga.on = 0;
+        if (G->p.flags == 0) vg::host::gather_setup(it.a, G->loc_alt, (size_t)G->g.nvox + 16);
+        // the merge writes through the grid's ring and sets what a pending
+        // re-centre brought in to unknown
+        it.a.ring = ring_of(G);
+        G->pend_on = false;
         if (G->p.vox_inf == 0) it.a.pl.occ_inf = it.a.pl.occ_raw;
         it.a.occ_test = it.a.pl.occ_inf;
         it.dtype = f.dtype;
@@ -934,21 +939,29 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
         it.txw = G->g.wx % 8 == 0 ? 8 : 4;
         it.tz = B->inflate_tz;
         it.mwpu = B->merge_words;
-        it.tiles[0] = (G->g.wx + it.txw - 1) / it.txw;
-        it.tiles[1] = (G->g.ny + 7) / 8;
-        it.tiles[2] = (G->g.nz + it.tz - 1) / it.tz;
+        const vg::WordBox &box = it.a.box;
+        const int32_t lo[3] = {box.w0, box.y0, box.z0}, num[3] = {box.nw, box.ny, box.nz}, size[3] = {it.txw, 8, it.tz};
+        for (int k = 0; k < 3; ++k) {
+            it.tile0[k] = lo[k] / size[k];
+            it.tiles[k] = (lo[k] + num[k] + size[k] - 1) / size[k] - it.tile0[k];
+        }
         it.buffered = G->g.words < vg::kRunWords ? 1 : 0;
         const int64_t npix = (int64_t)f.width * f.height;
         const int64_t nrays = (2 * (int64_t)G->hw + 1) * (2 * (int64_t)G->hh + 1);
-        int64_t units[4] = {
-            ((npix + 3) / 4 + 255) / 256,
-            G->p.vox_inf > 0 ? (int64_t)it.tiles[0] * it.tiles[1] * it.tiles[2] : 0,
-            (nrays + (256 / it.lpr) - 1) / (256 / it.lpr),
-            (G->g.words + it.mwpu - 1) / it.mwpu};
-        // the merge writes through the grid's ring and sets what a pending
-        // re-centre brought in to unknown
-        it.a.ring = ring_of(G);
-        G->pend_on = false;
+        it.pix_units = (int32_t)(((npix + 3) / 4 + 255) / 256);
+        int64_t units[6] = {it.pix_units, G->p.vox_inf > 0 ? (int64_t)it.tiles[0] * it.tiles[1] * it.tiles[2] : 0};
+        if (it.a.ga.on) {
+            it.near_units = vg::gather::near_units_of(it.a);
+            it.skin_units = (int32_t)vg::gather::word_units<256, 1>(box);
+            it.box_units = (int32_t)vg::gather::word_units<vg::kBatchGatherWords, 4>(box);
+            units[0] += (vg::gather::table_threads(it.a) + 255) / 256;
+            units[3] = it.box_units + vg::gather::slab_units(it.a, 256);
+            units[4] = it.near_units + it.skin_units;
+            units[5] = vg::gather::late_units(it.a);
+        } else {
+            units[2] = (nrays + (256 / it.lpr) - 1) / (256 / it.lpr);
+            units[3] = (G->g.words + it.mwpu - 1) / it.mwpu;
+        }
         if (f.recentre) {
             // the ring moves now; what the re-centre brings in is left
             // pending, for the grid's next merge (or read)
@@ -962,7 +975,7 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
                 std::memcpy(G->origin, o2, sizeof(o2));
             }
         }
-        for (int p = 0; p < 4; ++p) {
+        for (int p = 0; p < 6; ++p) {
             it.off[p] = total[p];
             total[p] += units[p];
         }
@@ -973,7 +986,7 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
     // than others, so each frame's rays are spread over proportionally more
     // (partly filled) units: G_i = ceil(groups_i * rounds * blocks / T)
     // (unless the spread is tuned off).
-    if (B->spread == 1) {
+    if (B->spread == 1 && total[2]) {
         const int64_t T = total[2];
         const int64_t nb = batch_blocks(B);
         if (nb < 1) return VG_ECUDA;
@@ -1000,7 +1013,7 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
     ctl->wtotal3 = wtotal;
     ctl->bar_ns = B->bar_ns;
     ctl->bar_extra = B->bar_extra;
-    for (int p = 0; p < 4; ++p) ctl->total[p] = total[p];
+    for (int p = 0; p < 6; ++p) ctl->total[p] = total[p];
     B->bytes = sizeof(vg::BatchCtl) + (size_t)n * sizeof(vg::BatchItem);
     B->prepared = true;
     return VG_OK;

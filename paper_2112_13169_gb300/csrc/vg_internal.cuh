@@ -157,8 +157,10 @@ constexpr int32_t kLitRaysLast = 2;     // resolve: free > traced > occupied
 // units in each phase.
 struct BatchItem {
     FrameArgs a;
-    int64_t off[4];     // first unit of this frame in phases 1..4
-    int32_t tiles[3];   // inflate tile grid (x words / txw, y / 8, z / 8)
+    int64_t off[6];     // first unit of this frame in phases 1..4; 4, 5: in the gathered phases 3 and 3b
+    int32_t tiles[3];   // inflate tiles of the frame's box (x words / txw, y / 8, z / tz)
+    int32_t tile0[3];   // the first of them
+    int32_t pix_units;  // phase 1: units of pixels; the others write the ray table
     int32_t dtype;      // 0 f32, 1 u16
     int32_t vec;        // depth base aligned for 4-pixel loads
     int32_t lpr;        // K3 lanes per ray: 8, 16 or 32
@@ -166,8 +168,9 @@ struct BatchItem {
     int32_t tz;         // inflate tile height in slices: 4 or 8
     int32_t mwpu;       // plane words per phase-4 unit: 256 or 512
     int32_t buffered;   // packed runs fit (plane words < kRunWords)
-    int32_t near_units; // gathered form: phase-3 units that mark the voxels around the camera
-    int32_t pad;
+    int32_t near_units; // gathered phase 3: units that mark the voxels around the camera; then skin_units
+    int32_t skin_units;
+    int32_t box_units;  // gathered phase 4: units of the frame's box; the others clear slabs
     int64_t woff3;      // phase 3: weight of the units before this frame's
     int64_t w3;         // phase 3: weight of each of this frame's units
 };
@@ -176,12 +179,14 @@ struct BatchItem {
 // pending re-centre, unless tuned (other frames' units are 256 words, one
 // per thread).
 constexpr int kBatchMergeWords = 512;
+// Plane words per phase-4 unit of a gathered frame of a batch.
+constexpr int kBatchGatherWords = 128;
 
 // Control block of a batch launch, copied to the device with the items.
 struct BatchCtl {
     int32_t n;          // frames
     int32_t pad0;
-    int64_t total[4];   // units per phase
+    int64_t total[6];   // units per phase, as BatchItem::off
     unsigned bar_count; // grid barrier: arrivals
     unsigned bar_gen;   // grid barrier: generation
     unsigned error;     // set when a barrier wait ran out
