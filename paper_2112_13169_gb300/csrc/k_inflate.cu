@@ -49,14 +49,15 @@ __device__ __forceinline__ uint32_t smem_addr(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-template <int R, int TXW, int TY, int TZ>
-__host__ __device__ constexpr int tma_box_words() { return (TXW + 8) * (TY + 2 * R) * (TZ + 2 * R); }
+template <int TXW, int TY, int TZ>
+__host__ __device__ constexpr int tma_box_words(int r) { return (TXW + 8) * (TY + 2 * r) * (TZ + 2 * r); }
 
 template <int R, int TXW, int TY, int TZ>
 __global__ void __launch_bounds__(256) k_inflate_tma(const __grid_constant__ CUtensorMap tm, const PlaneGeom g,
-                                                     uint32_t *__restrict__ out, const int3 first) {
-    constexpr int BW = TXW + 8, HY = TY + 2 * R, HZ = TZ + 2 * R;
-    constexpr uint32_t kBytes = (uint32_t)tma_box_words<R, TXW, TY, TZ>() * 4u;
+                                                     uint32_t *__restrict__ out, const int r_rt, const int3 first) {
+    constexpr int BW = TXW + 8;
+    const int r = R > 0 ? R : r_rt;
+    const uint32_t bytes = (uint32_t)tma_box_words<TXW, TY, TZ>(r) * 4u;
     extern __shared__ __align__(128) uint32_t sm[];   // the box, then the x pass's HZ * HY * TXW words
     __shared__ __align__(8) uint64_t bar;
     pdl_trigger();
@@ -69,8 +70,8 @@ __global__ void __launch_bounds__(256) k_inflate_tma(const __grid_constant__ CUt
     __syncthreads();
     pdl_wait();   // occ_raw is K1's
     if (threadIdx.x == 0) {
-        const int x = tx * TXW - 4, y = ty * TY - R, z = tz * TZ - R;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(kBytes) : "memory");
+        const int x = tx * TXW - 4, y = ty * TY - r, z = tz * TZ - r;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
         asm volatile(
             "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
             ::"r"(smem_addr(sm)), "l"(reinterpret_cast<uint64_t>(&tm)), "r"(x), "r"(y), "r"(z), "r"(b)
@@ -88,7 +89,7 @@ __global__ void __launch_bounds__(256) k_inflate_tma(const __grid_constant__ CUt
         return;
     }
     // the word w0 - 1 of each staged row is column 3 of the box
-    units::inflate_passes<R, TXW, TY, TZ>(g, out, R, tx, ty, tz, sm, BW, 3, sm + BW * HY * HZ);
+    units::inflate_passes<R, TXW, TY, TZ>(g, out, r, tx, ty, tz, sm, BW, 3, sm + tma_box_words<TXW, TY, TZ>(r));
 }
 
 // The tiles of the frame's box: the first one and how many each way.
@@ -178,11 +179,11 @@ bool plane_map(const void *base, const PlaneGeom &g, int bw, int hy, int hz, CUt
 template <int R, int TXW, int TY, int TZ>
 cudaError_t run_tma(const FrameArgs &a, cudaStream_t s) {
     CUtensorMap m;
-    if (!plane_map(a.pl.occ_raw, a.g, TXW + 8, TY + 2 * R, TZ + 2 * R, m)) return run<R, TXW, TY, TZ>(a, s);
+    if (!plane_map(a.pl.occ_raw, a.g, TXW + 8, TY + 2 * a.r, TZ + 2 * a.r, m)) return run<R, TXW, TY, TZ>(a, s);
     int3 t0;
     const dim3 grid = box_tiles<TXW, TY, TZ>(a.box, t0);
-    const size_t bytes = sizeof(uint32_t) * (tma_box_words<R, TXW, TY, TZ>() + (TZ + 2 * R) * (TY + 2 * R) * TXW);
-    return launch_pdl(k_inflate_tma<R, TXW, TY, TZ>, grid, 256, bytes, s, m, a.g, a.pl.occ_inf, t0);
+    const size_t bytes = sizeof(uint32_t) * (tma_box_words<TXW, TY, TZ>(a.r) + (TZ + 2 * a.r) * (TY + 2 * a.r) * TXW);
+    return launch_pdl(k_inflate_tma<R, TXW, TY, TZ>, grid, 256, bytes, s, m, a.g, a.pl.occ_inf, a.r, t0);
 }
 
 template <int TXW, int TZ>
@@ -191,7 +192,12 @@ cudaError_t run_r(const FrameArgs &a, cudaStream_t s, bool tma) {
     case 1: return tma ? run_tma<1, TXW, 8, TZ>(a, s) : run<1, TXW, 8, TZ>(a, s);
     case 2: return tma ? run_tma<2, TXW, 8, TZ>(a, s) : run<2, TXW, 8, TZ>(a, s);
     case 3: return tma ? run_tma<3, TXW, 8, TZ>(a, s) : run<3, TXW, 8, TZ>(a, s);
-    default: return run<0, TXW, 8, 8>(a, s);   // other radii: 8-slice tiles, the radius at run time
+    default:
+        // other radii: 8-slice tiles, the radius at run time.  Radius 8 on a
+        // 200 x 200 x 100 grid (a frame's box of it): 9.4 us (16.6 on the whole
+        // grid with tiles staged by threads and 2r + 1 loads an output);
+        // radius 5 on 500 x 500 x 150: 13.0 (33.2; 21.3 on the box)
+        return tma ? run_tma<0, TXW, 8, 8>(a, s) : run<0, TXW, 8, 8>(a, s);
     }
 }
 
@@ -211,12 +217,12 @@ int sms_of_current_device() {
 }  // namespace
 
 cudaError_t configure_inflate() {
-    // the runtime-radius tile at vox_inf 15 needs about 104 KB of shared memory
-    cudaError_t e = cudaFuncSetAttribute(k_inflate<0, 4, 8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         160 * 1024);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_inflate<0, 8, 8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 160 * 1024);
+    // the runtime-radius tile at vox_inf 15 needs up to 135 KB of shared memory
+    const cudaFuncAttribute smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(k_inflate<0, 4, 8, 8>, smem, 160 * 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_inflate<0, 8, 8, 8>, smem, 160 * 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_inflate_tma<0, 4, 8, 8>, smem, 160 * 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_inflate_tma<0, 8, 8, 8>, smem, 160 * 1024);
     return e;
 }
 

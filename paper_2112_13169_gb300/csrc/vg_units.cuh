@@ -209,7 +209,8 @@ __host__ __device__ constexpr size_t inflate_smem_words(int r) {
 // st[(lz * hy + ly) * sx + ox + lx], lx in [0, TXW + 2), with zeros outside
 // the grid.  buf1 (hz * hy * TXW words) must not overlap the staged words;
 // the y pass reuses the staged words' memory.  CTA-cooperative (256
-// threads); ends with a barrier.
+// threads); ends with a barrier.  R > 0 is the radius, known to the compiler
+// (1 to 3); R == 0 takes r_rt (4 or more).
 template <int R, int TXW, int TY, int TZ>
 __device__ __forceinline__ void inflate_passes(const PlaneGeom &g, uint32_t *out, const int r_rt, int tile_x,
                                                int tile_y, int tile_z, uint32_t *st, int sx, int ox, uint32_t *buf1) {
@@ -229,8 +230,45 @@ __device__ __forceinline__ void inflate_passes(const PlaneGeom &g, uint32_t *out
     }
     __syncthreads();
 
-    // y pass into the staged words' memory (now free): hz * TY * TXW
     uint32_t *buf2 = st;
+    if (R == 0) {
+        // a radius of 4 to 15, at run time.  A window of 2r + 1 rows costs as
+        // many loads an output, so threads share them: the TY (8) outputs of a
+        // column have rows 7 .. 2r in common, and the rest is running ORs from
+        // either end (2r + 8 loads for 8 outputs); in z two outputs share
+        // all rows but one each.
+        for (int i = threadIdx.x; i < hz * TXW; i += 256) {
+            const uint32_t *b = buf1 + (i / TXW) * hy * TXW + i % TXW;
+            uint32_t low[TY], mid = 0, up = 0;   // low[y]: rows y .. 6
+            low[TY - 1] = 0;
+#pragma unroll
+            for (int y = TY - 2; y >= 0; --y) low[y] = low[y + 1] | b[y * TXW];
+#pragma unroll 4
+            for (int y = TY - 1; y <= 2 * r; ++y) mid |= b[y * TXW];
+            uint32_t *o = buf2 + (i / TXW) * TY * TXW + i % TXW;
+#pragma unroll
+            for (int y = 0; y < TY; ++y) {
+                if (y) up |= b[(2 * r + y) * TXW];
+                o[y * TXW] = low[y] | mid | up;
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < TZ / 2 * TY * TXW; i += 256) {
+            const int c = i % (TY * TXW), lz = i / (TY * TXW) * 2, lx = c % TXW;
+            const uint32_t *b = buf2 + lz * TY * TXW + c;
+            uint32_t mid = 0;
+#pragma unroll 4
+            for (int d = 1; d <= 2 * r; ++d) mid |= b[d * TY * TXW];
+            const int w = w0 + lx, y = y0 + c / TXW, z = z0 + lz;
+            if (w >= g.wx || y >= g.ny) continue;
+            if (z < g.nz) out[((int64_t)z * g.ny + y) * g.wx + w] = mid | b[0];
+            if (z + 1 < g.nz) out[((int64_t)(z + 1) * g.ny + y) * g.wx + w] = mid | b[(2 * r + 1) * TY * TXW];
+        }
+        __syncthreads();   // the tile's shared memory may be reused right away
+        return;
+    }
+
+    // y pass into the staged words' memory (now free): hz * TY * TXW
     const int n2 = hz * TY * TXW;
     for (int i = threadIdx.x; i < n2; i += 256) {
         const int lx = i % TXW, rest = i / TXW, ly = rest % TY, lz = rest / TY;
