@@ -161,15 +161,20 @@ __device__ __forceinline__ void voxelize_depth_thread(const FrameArgs &a, int64_
     count_points(a, kept);
 }
 
+// The word and bit of point i of the cloud (kNoWord past its end).
+__device__ __forceinline__ uint32_t point_of_cloud(const FrameArgs &a, int64_t i, uint32_t &bit) {
+    if (i >= a.npts) return kNoWord;
+    const float x = __ldg(a.xyz + 3 * i + 0);
+    const float y = __ldg(a.xyz + 3 * i + 1);
+    const float z = __ldg(a.xyz + 3 * i + 2);
+    if (!(isfinite(x) && isfinite(y) && isfinite(z))) return kNoWord;
+    return point_word(a, x, y, z, bit);
+}
+
 // Point i of the cloud.  Warp-synchronous like voxelize_depth_thread.
 __device__ __forceinline__ void voxelize_points_thread(const FrameArgs &a, int64_t i) {
-    uint32_t key = kNoWord, bit = 0;
-    if (i < a.npts) {
-        const float x = __ldg(a.xyz + 3 * i + 0);
-        const float y = __ldg(a.xyz + 3 * i + 1);
-        const float z = __ldg(a.xyz + 3 * i + 2);
-        if (isfinite(x) && isfinite(y) && isfinite(z)) key = point_word(a, x, y, z, bit);
-    }
+    uint32_t bit = 0;
+    const uint32_t key = point_of_cloud(a, i, bit);
     warp_set_bits(a.pl.occ_raw, key, bit);
     count_points(a, key != kNoWord);
 }
