@@ -214,7 +214,8 @@ int stage_input(vg_grid *G, const void *src, size_t bytes, cudaStream_t s, const
 }
 
 FrameArgs frame_args(vg_grid *G, const vg::Pose32 &T) {
-    FrameArgs a = vg::host::frame_args(&G->p, G->g, T);
+    const int32_t bundle[3] = {G->vd, G->hw, G->hh};
+    FrameArgs a = vg::host::frame_args(&G->p, G->g, T, bundle);
     a.pl = G->pl;
     a.loc = G->loc;
     a.stats = (G->p.flags & VG_FLAG_STATS) ? G->stats : nullptr;

@@ -118,20 +118,27 @@ inline bool depth_frame_ok(int32_t width, int32_t height, int32_t dtype, float d
 
 // The kernel arguments of one measurement of a grid with parameters p and
 // plane geometry g (planes, loc and stats are left for the caller).
-inline FrameArgs frame_args(const vg_params *p, const PlaneGeom &g, const Pose32 &T) {
+// bundle: {vox_depth, hw, hh} where the caller has them.
+inline FrameArgs frame_args(const vg_params *p, const PlaneGeom &g, const Pose32 &T, const int32_t *bundle = nullptr) {
     FrameArgs a;
     std::memset(&a, 0, sizeof(a));
     a.g = g;
     a.T = T;
     a.vs = p->vox_size;
     a.depth_max = p->depth;
-    bundle_of(p, a.vd, a.hw, a.hh);
+    if (bundle) {
+        a.vd = bundle[0];
+        a.hw = bundle[1];
+        a.hh = bundle[2];
+    } else {
+        bundle_of(p, a.vd, a.hw, a.hh);
+    }
     a.r = p->vox_inf;
     a.box = {0, g.wx, 0, g.ny, 0, g.nz};
     return a;
 }
 
-inline void depth_box(FrameArgs &a, const vg_params *p);
+inline void depth_box(FrameArgs &a, const vg_params *p, double tx, double ty);
 
 // Adds a depth frame's input and pinhole intrinsics to a.
 inline void set_depth_frame(FrameArgs &a, const vg_params *p, const void *depth, int32_t width, int32_t height,
@@ -140,21 +147,22 @@ inline void set_depth_frame(FrameArgs &a, const vg_params *p, const void *depth,
     a.W = width;
     a.H = height;
     a.scale = (dtype == VG_DEPTH_U16) ? depth_scale : 1.0f;
-    a.fx = (float)(((double)width / 2.0) / tan(half_fov(p->fov_x_deg)));
-    a.fy = (float)(((double)height / 2.0) / tan(half_fov(p->fov_y_deg)));
+    const double tx = tan(half_fov(p->fov_x_deg)), ty = tan(half_fov(p->fov_y_deg));
+    a.fx = (float)(((double)width / 2.0) / tx);
+    a.fy = (float)(((double)height / 2.0) / ty);
     a.cx = (float)(((double)width - 1.0) / 2.0);
     a.cy = (float)(((double)height - 1.0) / 2.0);
-    depth_box(a, p);
+    depth_box(a, p, tx, ty);
 }
 
 // Narrows a depth frame's box to what its pixels (inflated by vox_inf) and
 // rays can reach: the pyramid of both from the camera, with two voxels to
-// spare for rounding.  Poses whose rotation block is no rotation keep their
+// spare for rounding (tx, ty: the tangents of half its fields of view).  Poses whose rotation block is no rotation keep their
 // linear map, so the corners bound it all the same.
-inline void depth_box(FrameArgs &a, const vg_params *p) {
+inline void depth_box(FrameArgs &a, const vg_params *p, double tx, double ty) {
     const double d = std::max((double)a.vd, (double)p->depth / (double)p->vox_size);
-    const double kx = std::max(tan(half_fov(p->fov_x_deg)), a.vd > 0 ? (double)a.hw / a.vd : 0.0) * d;
-    const double ky = std::max(tan(half_fov(p->fov_y_deg)), a.vd > 0 ? (double)a.hh / a.vd : 0.0) * d;
+    const double kx = std::max(tx, a.vd > 0 ? (double)a.hw / a.vd : 0.0) * d;
+    const double ky = std::max(ty, a.vd > 0 ? (double)a.hh / a.vd : 0.0) * d;
     int32_t lo[3], hi[3];
     const int32_t n[3] = {a.g.nx, a.g.ny, a.g.nz};
     for (int k = 0; k < 3; ++k) {

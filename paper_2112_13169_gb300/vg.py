@@ -199,6 +199,8 @@ def _stream(stream):
     """The cudaStream_t (an integer) to pass for `stream`."""
     global _CUDA, _CURRENT_STREAM
     if stream is None:
+        if _CURRENT_STREAM is not None:
+            return _CURRENT_STREAM()
         if _CUDA is None:
             t = _torch()
             _CUDA = bool(t is not None and t.cuda.is_available())
@@ -212,12 +214,12 @@ def _stream(stream):
 
 def _buffer(x):
     """(pointer, mem kind, nbytes, dtype string) of a tensor or array."""
-    t = _torch()
+    t = _TORCH or _torch()
     if t is not None and isinstance(x, t.Tensor):
         if not x.is_contiguous():
             raise ValueError("buffer must be contiguous")
         dt = _TORCH_DTYPES.get(x.dtype) or str(x.dtype).replace("torch.", "")
-        return x.data_ptr(), (VG_MEM_DEVICE if x.is_cuda else VG_MEM_HOST), x.numel() * x.element_size(), dt
+        return x.data_ptr(), (VG_MEM_DEVICE if x.is_cuda else VG_MEM_HOST), x.nbytes, dt
     a = x
     if not (isinstance(a, np.ndarray) and a.flags.c_contiguous):
         raise ValueError("buffer must be a contiguous numpy array or torch tensor")
@@ -225,16 +227,15 @@ def _buffer(x):
 
 
 def _f64(v, n):
-    """(array, pointer) of v as n contiguous float64 values; the array must
-    outlive the call that uses the pointer."""
-    if type(v) is np.ndarray and v.dtype is _F64 and v.size == n and v.flags.c_contiguous:
-        a = v
-    else:
-        a = np.ascontiguousarray(np.asarray(v, dtype=np.float64).reshape(n))
-    return a, a.__array_interface__["data"][0]
+    """v as n contiguous float64 values in a bytes object, which ctypes passes
+    as a pointer (asking an array for its address costs more than the copy)."""
+    if type(v) is np.ndarray and v.dtype is _F64 and v.size == n:
+        return v.tobytes()
+    return np.asarray(v, dtype=np.float64).reshape(n).tobytes()
 
 
 _F64 = np.dtype(np.float64)
+_Origin = C.c_int32 * 3
 _DEPTH_DTYPES = {"float32": VG_DEPTH_F32, "uint16": VG_DEPTH_U16}
 
 
@@ -257,8 +258,7 @@ def vg_ray_bundle(params):
 
 def vg_create(params, robot_pos_w, stream=None):
     h = C.c_void_p()
-    pos, pp = _f64(robot_pos_w, 3)
-    _check(load().vg_create(C.byref(params), pp, _stream(stream), C.byref(h)), "vg_create")
+    _check(load().vg_create(C.byref(params), _f64(robot_pos_w, 3), _stream(stream), C.byref(h)), "vg_create")
     return h
 
 
@@ -271,9 +271,9 @@ def vg_integrate_depth(h, depth, T_wc, depth_scale=1.0, stream=None):
     ptr, mem, nbytes, dt = _buffer(depth)
     dtype = _depth_dtype(dt)
     H, W = depth.shape
-    T, tp = _f64(T_wc, 16)
-    _check((_LIB or load()).vg_integrate_depth(h, ptr, mem, W, H, dtype, depth_scale, tp, _stream(stream)),
-           "vg_integrate_depth")
+    rc = (_LIB or load()).vg_integrate_depth(h, ptr, mem, W, H, dtype, depth_scale, _f64(T_wc, 16), _stream(stream))
+    if rc:
+        _check(rc, "vg_integrate_depth")
 
 
 def vg_integrate_depth_noalloc(params, origin, loc, depth, T_wc, depth_scale=1.0, stream=None):
@@ -294,7 +294,7 @@ def vg_integrate_depth_noalloc(params, origin, loc, depth, T_wc, depth_scale=1.0
     dtype = _depth_dtype(dt)
     H, W = depth.shape
     o = np.ascontiguousarray(np.asarray(origin, np.int32).reshape(3))
-    T, tp = _f64(T_wc, 16)
+    tp = _f64(T_wc, 16)
     t = _torch()
     # the library runs on the current device: make it loc's
     with t.cuda.device(loc.device):
@@ -307,21 +307,25 @@ def vg_integrate_points(h, xyz, T_wc, stream=None):
     ptr, mem, nbytes, dt = _buffer(xyz)
     if dt != "float32":
         raise ValueError("points must be float32 xyz triples")
-    T, tp = _f64(T_wc, 16)
-    _check(load().vg_integrate_points(h, ptr, mem, nbytes // 12, tp, _stream(stream)), "vg_integrate_points")
+    rc = (_LIB or load()).vg_integrate_points(h, ptr, mem, nbytes // 12, _f64(T_wc, 16), _stream(stream))
+    if rc:
+        _check(rc, "vg_integrate_points")
 
 
 def vg_shift(h, robot_pos_w, stream=None):
-    pos, pp = _f64(robot_pos_w, 3)
-    _check((_LIB or load()).vg_shift(h, pp, _stream(stream)), "vg_shift")
+    rc = (_LIB or load()).vg_shift(h, _f64(robot_pos_w, 3), _stream(stream))
+    if rc:
+        _check(rc, "vg_shift")
 
 
 def vg_read(h, dst, stream=None):
     """Enqueue a copy of loc_grid into dst; returns the origin (int32[3])."""
     ptr, mem, nbytes, _ = _buffer(dst)
-    o = np.zeros(3, np.int32)
-    _check((_LIB or load()).vg_read(h, ptr, mem, nbytes, o.ctypes.data, _stream(stream)), "vg_read")
-    return o
+    o = _Origin()
+    rc = (_LIB or load()).vg_read(h, ptr, mem, nbytes, o, _stream(stream))
+    if rc:
+        _check(rc, "vg_read")
+    return np.frombuffer(o, np.int32)
 
 
 def vg_write(h, src, origin, stream=None):
@@ -412,7 +416,7 @@ class Grid:
         ptr, mem, nbytes, dt = _buffer(depth)
         dtype = _depth_dtype(dt)
         H, W = depth.shape
-        T, tp = _f64(T_wc, 16)
+        tp = _f64(T_wc, 16)
         best = (C.c_int32 * 6)()
         _check(load().vg_autotune(self.h, ptr, mem, W, H, dtype, float(depth_scale), tp, int(reps), _stream(stream),
                                   best), "vg_autotune")
@@ -450,12 +454,10 @@ def make_frames(frames):
         fr.width, fr.height = int(W), int(H)
         fr.dtype = VG_DEPTH_F32 if dt == "float32" else VG_DEPTH_U16
         fr.depth_scale = float(scale)
-        T, tp = _f64(T_wc, 16)
-        C.memmove(fr.T_wc, tp, 128)
+        C.memmove(fr.T_wc, _f64(T_wc, 16), 128)
         if pos is not None:
             fr.recentre = 1
-            P, pp = _f64(pos, 3)
-            C.memmove(fr.robot_pos_w, pp, 24)
+            C.memmove(fr.robot_pos_w, _f64(pos, 3), 24)
     return arr
 
 
@@ -524,8 +526,8 @@ class Server:
     def add_camera(self, n, vox_size, fov_x_deg, fov_y_deg, depth, vox_inf, robot_pos_w=(0, 0, 0)):
         params = make_params(n, vox_size, fov_x_deg, fov_y_deg, depth, vox_inf)
         cam = C.c_int32()
-        pos, pp = _f64(robot_pos_w, 3)
-        _check(load().vg_server_add_camera(self.h, C.byref(params), pp, C.byref(cam)), "vg_server_add_camera")
+        _check(load().vg_server_add_camera(self.h, C.byref(params), _f64(robot_pos_w, 3), C.byref(cam)),
+               "vg_server_add_camera")
         return int(cam.value)
 
     def remove_camera(self, camera):
@@ -539,8 +541,8 @@ class Server:
             raise ValueError("served frames come from host memory")
         dtype = _depth_dtype(dt)
         H, W = depth.shape
-        T, tp = _f64(T_wc, 16)
-        pos, pp = _f64(robot_pos_w if robot_pos_w is not None else (0.0, 0.0, 0.0), 3)
+        tp = _f64(T_wc, 16)
+        pp = _f64(robot_pos_w if robot_pos_w is not None else (0.0, 0.0, 0.0), 3)
         t = C.c_uint64()
         rc = load().vg_server_submit(self.h, int(camera), ptr, int(W), int(H), dtype, float(depth_scale), tp,
                                      1 if robot_pos_w is not None else 0, pp, C.byref(t))
