@@ -156,10 +156,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
                 continue;
             }
             switch (s_kind) {
-            case 0: units::voxelize_depth_thread<0, false>(s_a, t); break;
-            case 1: units::voxelize_depth_thread<0, true>(s_a, t); break;
-            case 2: units::voxelize_depth_thread<1, false>(s_a, t); break;
-            default: units::voxelize_depth_thread<1, true>(s_a, t); break;
+            case 0: units::voxelize_depth_thread<0, false, false>(s_a, t); break;
+            case 1: units::voxelize_depth_thread<0, true, false>(s_a, t); break;
+            case 2: units::voxelize_depth_thread<1, false, false>(s_a, t); break;
+            default: units::voxelize_depth_thread<1, true, false>(s_a, t); break;
             }
         }
     }

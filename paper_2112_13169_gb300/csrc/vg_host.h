@@ -116,6 +116,16 @@ inline bool depth_frame_ok(int32_t width, int32_t height, int32_t dtype, float d
     return true;
 }
 
+// 1 / y rounded to nearest, for K1's divisions by a constant (units::div_by),
+// or 0 where their correction step might not round correctly: y far from 1,
+// or with a significand of all ones.
+inline float reciprocal(float y) {
+    uint32_t bits;
+    std::memcpy(&bits, &y, sizeof(bits));
+    if (!(y >= 1e-18f && y <= 1e18f) || (bits & 0x7fffffu) == 0x7fffffu) return 0.0f;
+    return 1.0f / y;
+}
+
 // The kernel arguments of one measurement of a grid with parameters p and
 // plane geometry g (planes, loc and stats are left for the caller).
 // bundle: {vox_depth, hw, hh} where the caller has them.
@@ -125,6 +135,7 @@ inline FrameArgs frame_args(const vg_params *p, const PlaneGeom &g, const Pose32
     a.g = g;
     a.T = T;
     a.vs = p->vox_size;
+    a.rvs = reciprocal(a.vs);
     a.depth_max = p->depth;
     if (bundle) {
         a.vd = bundle[0];
@@ -150,6 +161,8 @@ inline void set_depth_frame(FrameArgs &a, const vg_params *p, const void *depth,
     const double tx = tan(half_fov(p->fov_x_deg)), ty = tan(half_fov(p->fov_y_deg));
     a.fx = (float)(((double)width / 2.0) / tx);
     a.fy = (float)(((double)height / 2.0) / ty);
+    a.rfx = reciprocal(a.fx);
+    a.rfy = reciprocal(a.fy);
     a.cx = (float)(((double)width - 1.0) / 2.0);
     a.cy = (float)(((double)height - 1.0) / 2.0);
     depth_box(a, p, tx, ty);

@@ -132,6 +132,7 @@ struct FrameArgs {
     int32_t W, H;
     float scale;       // u16 -> metres
     float fx, fy, cx, cy;
+    float rvs, rfx, rfy;        // reciprocals for K1's divisions (host::reciprocal)
     // point cloud input
     const float *xyz;
     int64_t npts;
