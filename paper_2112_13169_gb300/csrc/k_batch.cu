@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
                 const int32_t box = __ldg(&it.box_units);
                 if (local < box) {
                     gather::frame_start(s_a, S, v0);
-                    gather::gather_unit<kGatherWords, units::LoadPlain>(
+                    gather::gather_unit<kGatherWords, false, units::LoadPlain>(
                         s_a, S, v0, (uint32_t)local, box, *reinterpret_cast<gather::GatherSmem<kGatherWords> *>(dyn));
                 } else {
                     gather::slab_word(s_a, (local - box) * kThreads + threadIdx.x);

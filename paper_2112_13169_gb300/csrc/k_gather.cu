@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(kThreads) k_gather(const FrameArgs a, const in
     int32_t v0[3];
     frame_start(a, S, v0);
     pdl_wait();
-    if ((int)blockIdx.x < nbox) gather_unit<WPU, units::LoadPlain>(a, S, v0, blockIdx.x, nbox, sh);
+    if ((int)blockIdx.x < nbox) gather_unit<WPU, true, units::LoadPlain>(a, S, v0, blockIdx.x, nbox, sh);
     else slab_word(a, (int64_t)((int)blockIdx.x - nbox) * kThreads + threadIdx.x);
 }
 
@@ -67,7 +67,7 @@ cudaError_t launch_rayhit(const FrameArgs &a, cudaStream_t s) {
 // 76 k 44 / 41 / 47, of 200 k 83 / 77 / 77, of 600 k 203 / 174 / 163.
 cudaError_t launch_gather(const FrameArgs &a, cudaStream_t s) {
     const int64_t words = (int64_t)a.box.nw * a.box.ny * a.box.nz;
-    if (words < 55000) return gather_words<64>(a, s);
+    if (words < 45000) return gather_words<64>(a, s);
     if (words < 250000) return gather_words<128>(a, s);
     return gather_words<256>(a, s);
 }

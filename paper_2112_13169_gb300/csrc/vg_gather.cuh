@@ -53,12 +53,15 @@
 
 #include "vg_units.cuh"
 
+#include <type_traits>
+
 namespace vg {
 namespace gather {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kThreads = 256;
 constexpr uint32_t kNoHit = 0xffffffffu;
+constexpr uint32_t kNone = 0xfffffffeu;   // no ray's key: no ray has a certain say
 constexpr int kNear = kNearReach, kNearN = 2 * kNear + 1, kNearRows = kNearWords;
 constexpr float kMargin = kGatherMargin;
 constexpr float kSphere = 0.46f;
@@ -575,17 +578,17 @@ __device__ __forceinline__ void late_unit(const FrameArgs &a, int32_t unit, Late
 // patch, and byte p of the four words of a group are patch p's rows, so thread
 // 4 g + p stands for word p and for patch p of group g.  Masks are kept as
 // bytes [word][patch].
-constexpr uint32_t kInside = 0x80000000u;
 template <int WPU>
 struct GatherSmem {
     uint32_t oc[WPU], need[WPU], fr[WPU], tr[WPU], ent[WPU];
     uint32_t at[WPU];          // the word's place: x word, y, z in 7, 12 and 12 bits
     Place first[WPU];          // the place of the patch's first voxel in camera axes
-    uint16_t list[WPU];        // patches inside the bundle; kInside's top half: well inside
+    uint32_t row[WPU];         // the first byte of the word's row in the ring-addressed loc_grid
+    uint16_t list[WPU];        // patches that touch the bundle: well inside; from the end: at its edges
     uint16_t open[WPU * 32];   // voxels to resolve: patch * 32 + voxel; from the end: those the nearest ray traces
     uint16_t hard[WPU * 32];   // voxels that take every ray of their windows
     PairSmem pairs;
-    uint32_t nlist, nlisted, nhard;   // nlisted: open ones, and from bit 16 those from the end
+    uint32_t nlist, nopen, nhard;   // the first two: entries, and from bit 16 those from the end
 };
 
 // Appends this lane's value to a list in shared memory if `in`; all lanes of
@@ -604,7 +607,11 @@ __device__ __forceinline__ void push(uint16_t *list, uint32_t *n, bool in, uint3
 // their codes through the ring (as merge_word does: unknown where a re-centre
 // brought the voxel in and nothing marks it) and clears the occupancy words.
 // CTA-cooperative.
-template <int WPU, class L>
+// SPLIT: patches well inside the bundle and at its edges are resolved by loops
+// of their own (a frame alone: 208 -> 193 us for three 1280x720 frames); the
+// fused batch, whose code is larger than the instruction cache likes, keeps
+// one (a step of 64 robots 550 us, 566 with two).
+template <int WPU, bool SPLIT, class L>
 __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3], const int32_t v0[3], uint32_t unit,
                                             uint32_t units, GatherSmem<WPU> &sh) {
     const Gather &g = a.ga;
@@ -612,7 +619,7 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
     const float fvd = (float)a.vd;
     if (tid == 0) {
         sh.nlist = 0;
-        sh.nlisted = 0;
+        sh.nopen = 0;
         sh.nhard = 0;
     }
     __syncthreads();
@@ -624,6 +631,8 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
         int32_t i[3];
         if (unit_word<4>(a, unit, units, i)) {
             const uint32_t w = word_of(a.g, i);
+            sh.row[tid] = (uint32_t)(units::ring_at(i[2], a.ring.r[2], a.g.nz) * a.g.ny +
+                                     units::ring_at(i[1], a.ring.r[1], a.g.ny)) * (uint32_t)a.g.nx;
             oc = L::ld(a.pl.occ_inf + w);
             const int nbits = min(32, a.g.nx - i[0]);
             const uint32_t valid = nbits >= 32 ? kFull : ((1u << nbits) - 1u);
@@ -660,7 +669,15 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
                             m.c2 - g.zp > 0.5f && m.c2 + g.zp < fvd;
         uint32_t some = need | __shfl_xor_sync(kFull, need, 1);   // the patch's columns, over its four rows
         some = ((some | __shfl_xor_sync(kFull, some, 2)) >> (8 * (tid & 3))) & 255u;
-        push(sh.list, &sh.nlist, in && some, (uint32_t)tid | (inside ? kInside >> 16 : 0u));
+        const unsigned mi = __ballot_sync(kFull, in && some && inside), me = __ballot_sync(kFull, in && some && !inside);
+        if (mi | me) {
+            uint32_t at = 0;
+            if (lane == 0) at = atomicAdd(&sh.nlist, (uint32_t)__popc(mi) + ((uint32_t)__popc(me) << 16));
+            at = __shfl_sync(kFull, at, 0);
+            const unsigned below = (1u << lane) - 1u;
+            if ((mi >> lane) & 1u) sh.list[(at & 0xffffu) + __popc(mi & below)] = (uint16_t)tid;
+            if ((me >> lane) & 1u) sh.list[WPU - 1 - (at >> 16) - __popc(me & below)] = (uint16_t)tid;
+        }
     }
     __syncthreads();
 
@@ -675,39 +692,43 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
     const int32_t width = 2 * a.hw + 1, centre = a.hh * width + a.hw;
     const uint32_t *hits = g.hit + centre;
     const uint32_t *latest = reinterpret_cast<const uint32_t *>(g.inv + centre) + 3;
-    const uint32_t nlist = sh.nlist;
-    for (uint32_t l0 = warp * kFlight; l0 < nlist; l0 += kThreads / 32 * kFlight) {
-        uint32_t patch[kFlight], hit[kFlight], late[kFlight];
+    const uint32_t kzr = __float_as_uint(fminf((g.zr - zmin) * ivd, 1.5f)) << 2;   // (1.5: never)
+    auto certain = [&](auto edge, uint32_t l0, uint32_t nlist) {
+        const bool kEdge = edge;
+        uint32_t patch[kFlight], hit[kFlight], late[kFlight], kmin[kFlight], kmid[kFlight];
         int32_t ray[kFlight];
-        float c2[kFlight];
         bool in[kFlight];
 #pragma unroll
         for (int k = 0; k < kFlight; ++k) {
-            const uint32_t le = sh.list[min(l0 + k, nlist - 1u)];
-            patch[k] = le & 0x7fffu;
+            const uint32_t l = min(l0 + k, nlist - 1u);
+            patch[k] = sh.list[kEdge ? WPU - 1 - l : l];
             const Place q = sh.first[patch[k]];
             const Place p = {q.c0 + o0, q.c1 + o1, q.c2 + o2};
             in[k] = l0 + k < nlist && (((uint32_t)need8[4u * ((patch[k] & ~3u) + (uint32_t)(lane >> 3)) + (patch[k] & 3u)] >> (lane & 7)) & 1u);
             bool ranged = in[k];
-            if (!(le & (kInside >> 16))) {
+            if (kEdge) {
                 in[k] = in[k] && in_bundle(a, p, g.ev, g.zv);
                 ranged = in[k] && p.c2 > 0.5f && p.c2 < fvd - kMargin;
             }
             // the nearest ray, its indices by adding 1.5 * 2^23
             const float z = __fdividef(fvd, p.c2), tau = p.c2 * ivd;
-            const float fa = fminf(fmaxf(p.c0 * z, -fw), fw), fb = fminf(fmaxf(p.c1 * z, -fh), fh);
+            float fa = p.c0 * z, fb = p.c1 * z;
+            if (kEdge) {
+                fa = fminf(fmaxf(fa, -fw), fw);
+                fb = fminf(fmaxf(fb, -fh), fh);
+            }
             const float ma = fa + 12582912.0f, mb = fb + 12582912.0f;
             const float da = __fmaf_rn(12582912.0f - ma, tau, p.c0), db = __fmaf_rn(12582912.0f - mb, tau, p.c1);
-            c2[k] = p.c2;
             ray[k] = (__float_as_int(mb) - 0x4b400000) * width + (__float_as_int(ma) - 0x4b400000);
-            hit[k] = 0xfffffffeu;   // no say
+            kmin[k] = __float_as_uint(fmaxf((p.c2 - zmin) * ivd, 0.0f)) << 2;
+            kmid[k] = __float_as_uint(tau) << 2 | 3u;
+            hit[k] = kNone;
             if (ranged && __fmaf_rn(da, da, db * db) < kSphere * kSphere) hit[k] = L::ld(hits + ray[k]);
         }
 #pragma unroll
         for (int k = 0; k < kFlight; ++k) {
             late[k] = kNoHit;
-            const uint32_t kmin = __float_as_uint(fmaxf((c2[k] - zmin) * ivd, 0.0f)) << 2;
-            if (hit[k] < kmin && c2[k] >= g.zr) late[k] = L::ld(latest + 4 * ray[k]);
+            if (hit[k] < kmin[k] && kmin[k] >= kzr) late[k] = L::ld(latest + 4 * ray[k]);
         }
         // free: the hit lies past the centre; traced: before the voxel's
         // nearest depth, and final unless some ray that reaches the voxel
@@ -716,9 +737,8 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
         uint32_t count = 0;   // of the open ones, and from bit 16 of those behind
 #pragma unroll
         for (int k = 0; k < kFlight; ++k) {
-            const uint32_t kmin = __float_as_uint(fmaxf((c2[k] - zmin) * ivd, 0.0f)) << 2;
-            const bool free = hit[k] != 0xfffffffeu && hit[k] > ((__float_as_uint(c2[k] * ivd) << 2) | 3u);
-            const bool behind = hit[k] < kmin, traced = late[k] < kmin;
+            const bool free = hit[k] != kNone && hit[k] > kmid[k];
+            const bool behind = hit[k] < kmin[k], traced = late[k] < kmin[k];
             const unsigned mf = __ballot_sync(kFull, free), mt = __ballot_sync(kFull, behind);
             mo[k] = __ballot_sync(kFull, in[k] && !free && !behind);
             mb[k] = __ballot_sync(kFull, behind && !traced);
@@ -732,7 +752,7 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
         }
         if (count) {
             uint32_t at = 0;
-            if (lane == 0) at = atomicAdd(&sh.nlisted, count);
+            if (lane == 0) at = atomicAdd(&sh.nopen, count);
             at = __shfl_sync(kFull, at, 0);
             const unsigned below = (1u << lane) - 1u;
             uint32_t po = at & 0xffffu, pb = WPU * 32 - 1 - (at >> 16);
@@ -743,6 +763,20 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
                 po += __popc(mo[k]);
                 pb -= __popc(mb[k]);
             }
+        }
+    };
+    const uint32_t nin = sh.nlist & 0xffffu, nedge = sh.nlist >> 16;
+    if (SPLIT) {
+        for (uint32_t l0 = warp * kFlight; l0 < nin; l0 += kThreads / 32 * kFlight)
+            certain(std::false_type(), l0, nin);
+        // (the other way round, so that the warps that had a round less begin)
+        for (uint32_t l0 = (kThreads / 32 - 1 - warp) * kFlight; l0 < nedge; l0 += kThreads / 32 * kFlight)
+            certain(std::true_type(), l0, nedge);
+    } else {
+        const uint32_t rounds = (nin + kFlight - 1) / kFlight, all = rounds + (nedge + kFlight - 1) / kFlight;
+        for (uint32_t l = warp; l < all; l += kThreads / 32) {
+            const bool edge = l >= rounds;
+            certain(edge, (edge ? l - rounds : l) * kFlight, edge ? nedge : nin);
         }
     }
     __syncthreads();
@@ -767,7 +801,7 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
     auto window = [&](uint32_t e) { return window_of(a, place(e), 0.5f, g.zv); };
 
     // ---- traced ones that a later hit of some ray in their window may free
-    const uint32_t nback = sh.nlisted >> 16, nopen = sh.nlisted & 0xffffu;
+    const uint32_t nback = sh.nopen >> 16, nopen = sh.nopen & 0xffffu;
     for (uint32_t l0 = warp * 32; l0 < nback; l0 += kThreads) {
         uint32_t e = 0;
         bool hard = false;
@@ -808,11 +842,16 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
             uint32_t E;
             voxel(e, i);
             hard = true;
-            if (visits(L::ld(g.inv + (centre + rb * width + ra)), S, v0, i, E)) {
+            const float4 v = L::ld(g.inv + (centre + rb * width + ra));
+            if (visits(v, S, v0, i, E)) {
+                // traced for good if no ray that reaches it hits later
+                const uint32_t kmin = __float_as_uint(fmaxf((p.c2 - zmin) * ivd, 0.0f)) << 2;
                 hard = E >= h;
+                const bool last = hard && kmin >= kzr && __float_as_uint(v.w) < kmin;
                 uint32_t bit;
                 const uint32_t slot = word_bit(e, bit);
                 atomicOr((hard ? sh.tr : sh.fr) + slot, bit);
+                hard = hard && !last;
             }
         }
         push(sh.hard, &sh.nhard, hard, e);
@@ -845,8 +884,7 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
         units::code_masks(oc >> s, f >> s, t >> s, hi, lo, known);
         const uint32_t code = units::merge4(hi, lo, known, 0, 0u);
         const uint32_t at = sh.at[slot];
-        uint8_t *rowp = a.loc + ((int64_t)units::ring_at((int32_t)((at >> 19) & 4095u), a.ring.r[2], a.g.nz) * a.g.ny +
-                                 units::ring_at((int32_t)((at >> 7) & 4095u), a.ring.r[1], a.g.ny)) * a.g.nx;
+        uint8_t *rowp = a.loc + sh.row[slot];
         const int32_t x = (int32_t)(at & 127u) * 32 + s, xb = units::ring_at(x, a.ring.r[0], a.g.nx);
         uint8_t *p = rowp + xb;
         if (touch == 15u && xb + 4 <= a.g.nx && (reinterpret_cast<uintptr_t>(p) & 3u) == 0) {
