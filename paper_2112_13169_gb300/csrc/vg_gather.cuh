@@ -36,15 +36,15 @@
 //
 // Certain cases.  With p the voxel's centre and M the inverse rotation,
 // M (p - S) = tau (a, b, vd) gives the voxel's place in the bundle.  If the
-// nearest ray passes the centre within kSphere voxels at the centre's
-// depth, it crosses the voxel's inscribed sphere on a chord of 0.3 voxels or
+// nearest ray passes the centre within 0.49 - m voxels at the centre's
+// depth, it crosses the voxel's inscribed sphere on a chord of 0.19 voxels or
 // more, which is far beyond the rounding of the crossing times
-// (gather_setup bounds the coordinates), so the walk visits the voxel; if its
+// (gather_setup bounds it by m), so the walk visits the voxel; if its
 // hit lies past the centre's depth the voxel is free; if its hit, and those
 // of all rays around it that may reach the voxel (late_unit), lie before the
 // voxel's nearest depth, it is traced.  All other voxels inside the bundle's sides are listed and
 // resolved by testing every ray of their window with visits(); windows and
-// culling leave a margin of kMargin voxels for rounding.
+// culling leave the margin m for rounding.
 //
 // Voxels within kNear of the camera's would have windows of thousands of
 // rays; there the rays mark the voxels they walk through (near_unit), 15
@@ -63,8 +63,6 @@ constexpr int kThreads = 256;
 constexpr uint32_t kNoHit = 0xffffffffu;
 constexpr uint32_t kNone = 0xfffffffeu;   // no ray's key: no ray has a certain say
 constexpr int kNear = kNearReach, kNearN = 2 * kNear + 1, kNearRows = kNearWords;
-constexpr float kMargin = kGatherMargin;
-constexpr float kSphere = 0.46f;
 constexpr int kFlight = 4;     // loads in flight per thread
 constexpr int kFaces = 4096;   // faces a round of K3 lists
 
@@ -159,7 +157,7 @@ __device__ __forceinline__ bool in_bundle(const FrameArgs &a, const Place &p, co
     const Gather &g = a.ga;
     return __fmaf_rn(-g.ka, p.c2, p.c0) <= e[0] && __fmaf_rn(-g.ka, p.c2, -p.c0) <= e[1] &&
            __fmaf_rn(-g.kb, p.c2, p.c1) <= e[2] && __fmaf_rn(-g.kb, p.c2, -p.c1) <= e[3] &&
-           p.c2 + z + kMargin >= 0.0f && p.c2 - z - kMargin <= (float)a.vd;
+           p.c2 + z + g.m >= 0.0f && p.c2 - z - g.m <= (float)a.vd;
 }
 
 struct Window {
@@ -175,7 +173,7 @@ __device__ __forceinline__ Window window_of(const FrameArgs &a, const Place &p, 
     const Gather &g = a.ga;
     const float fvd = (float)a.vd, fw = (float)a.hw, fh = (float)a.hh;
     Window w;
-    const float zn = p.c2 - z - kMargin;
+    const float zn = p.c2 - z - g.m;
     w.kmin = __float_as_uint(fminf(fmaxf(__fdividef(zn, fvd), 0.0f), 1.0f)) << 2;
     if (zn < 0.2f) {
         w.alo = -a.hw; w.ahi = a.hw; w.blo = -a.hh; w.bhi = a.hh;
@@ -186,7 +184,7 @@ __device__ __forceinline__ Window window_of(const FrameArgs &a, const Place &p, 
                      0.5f * (fabsf(__fmaf_rn(-k0, g.M[7], g.M[1])) + fabsf(__fmaf_rn(-k0, g.M[8], g.M[2])));
     const float h1 = hx * fabsf(__fmaf_rn(-k1, g.M[6], g.M[3])) +
                      0.5f * (fabsf(__fmaf_rn(-k1, g.M[7], g.M[4])) + fabsf(__fmaf_rn(-k1, g.M[8], g.M[5])));
-    const float wa = __fmaf_rn(h0 + kMargin, q, kMargin), wb = __fmaf_rn(h1 + kMargin, q, kMargin);
+    const float wa = __fmaf_rn(h0 + g.m, q, g.m), wb = __fmaf_rn(h1 + g.m, q, g.m);
     const float fa = k0 * fvd, fb = k1 * fvd;
     w.alo = (int32_t)ceilf(fmaxf(fa - wa, -fw));
     w.ahi = (int32_t)floorf(fminf(fa + wa, fw));
@@ -196,22 +194,22 @@ __device__ __forceinline__ Window window_of(const FrameArgs &a, const Place &p, 
 }
 
 // The window of the face of voxel i that a walk enters through along axis k:
-// the projections of its corners, kMargin beyond its edges.
+// the projections of its corners, the margin beyond its edges.
 __device__ __forceinline__ Window face_window(const FrameArgs &a, const float S[3], const int32_t v0[3],
                                               const int32_t i[3], int k) {
     const Gather &g = a.ga;
     const float fvd = (float)a.vd, fw = (float)a.hw, fh = (float)a.hh;
-    constexpr float kSpan = 1.0f + 2.0f * kMargin;
+    const float span = 1.0f + 2.0f * g.m;
     float r[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j)
-        r[j] = (j == k ? (float)(i[j] + (i[j] < v0[j])) : (float)i[j] - kMargin) - S[j];
+        r[j] = (j == k ? (float)(i[j] + (i[j] < v0[j])) : (float)i[j] - g.m) - S[j];
     const Place p = place_of(g, r[0], r[1], r[2]);
     const int k1 = k == 0 ? 1 : 0, k2 = k == 2 ? 1 : 2;
-    const float u0 = kSpan * g.M[k1], u1 = kSpan * g.M[3 + k1], u2 = kSpan * g.M[6 + k1];
-    const float w0 = kSpan * g.M[k2], w1 = kSpan * g.M[3 + k2], w2 = kSpan * g.M[6 + k2];
+    const float u0 = span * g.M[k1], u1 = span * g.M[3 + k1], u2 = span * g.M[6 + k1];
+    const float w0 = span * g.M[k2], w1 = span * g.M[3 + k2], w2 = span * g.M[6 + k2];
     Window w;
-    const float zn = p.c2 + fminf(u2, 0.0f) + fminf(w2, 0.0f) - kMargin;
+    const float zn = p.c2 + fminf(u2, 0.0f) + fminf(w2, 0.0f) - g.m;
     w.kmin = __float_as_uint(fminf(fmaxf(__fdividef(zn, fvd), 0.0f), 1.0f)) << 2;
     if (zn < 0.2f) {
         w.alo = -a.hw; w.ahi = a.hw; w.blo = -a.hh; w.bhi = a.hh;
@@ -227,7 +225,7 @@ __device__ __forceinline__ Window face_window(const FrameArgs &a, const float S[
         blo = fminf(blo, y * q);
         bhi = fmaxf(bhi, y * q);
     }
-    const float m = __fmaf_rn(2.5f * kMargin, __fdividef(fvd, zn), kMargin);
+    const float m = __fmaf_rn(2.5f * g.m, __fdividef(fvd, zn), g.m);
     w.alo = (int32_t)ceilf(fmaxf(alo - m, -fw));
     w.ahi = (int32_t)floorf(fminf(ahi + m, fw));
     w.blo = (int32_t)ceilf(fmaxf(blo - m, -fh));
@@ -685,7 +683,7 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
     const uint8_t *need8 = reinterpret_cast<const uint8_t *>(sh.need);
     uint8_t *fr8 = reinterpret_cast<uint8_t *>(sh.fr), *tr8 = reinterpret_cast<uint8_t *>(sh.tr);
     const float ivd = 1.0f / fvd, fw = (float)a.hw, fh = (float)a.hh;
-    const float zmin = g.zv + kMargin;
+    const float zmin = g.zv + g.m;
     const float lx = (float)(lane & 7), ly = (float)(lane >> 3);
     const float o0 = __fmaf_rn(ly, g.M[1], lx * g.M[0]), o1 = __fmaf_rn(ly, g.M[4], lx * g.M[3]),
                 o2 = __fmaf_rn(ly, g.M[7], lx * g.M[6]);
@@ -708,7 +706,7 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
             bool ranged = in[k];
             if (kEdge) {
                 in[k] = in[k] && in_bundle(a, p, g.ev, g.zv);
-                ranged = in[k] && p.c2 > 0.5f && p.c2 < fvd - kMargin;
+                ranged = in[k] && p.c2 > 0.5f && p.c2 < fvd - g.m;
             }
             // the nearest ray, its indices by adding 1.5 * 2^23
             const float z = __fdividef(fvd, p.c2), tau = p.c2 * ivd;
@@ -723,7 +721,7 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
             kmin[k] = __float_as_uint(fmaxf((p.c2 - zmin) * ivd, 0.0f)) << 2;
             kmid[k] = __float_as_uint(tau) << 2 | 3u;
             hit[k] = kNone;
-            if (ranged && __fmaf_rn(da, da, db * db) < kSphere * kSphere) hit[k] = L::ld(hits + ray[k]);
+            if (ranged && __fmaf_rn(da, da, db * db) < g.sphere2) hit[k] = L::ld(hits + ray[k]);
         }
 #pragma unroll
         for (int k = 0; k < kFlight; ++k) {

@@ -212,13 +212,19 @@ inline bool gather_pays(const FrameArgs &a) {
 // Sets up the gathered form of a frame (vg_gather.cuh) in `bytes` bytes of
 // device memory at base (256-byte aligned), or leaves it off: a.T, a.vs, the
 // bundle and the geometry are set.  The form needs a rotation (within 1e-3:
-// a voxel's inscribed sphere stays one), a bundle of at most 105 degrees (a wider one
-// crosses voxels outside the near words at depths where windows are huge) and
-// a camera, grid and range within 4096 voxels, so that float coordinates in
-// camera axes (off by at most about 4096 * 2^-22 * 10) stay well inside
-// kGatherMargin, and room for its tables: 20 bytes a ray, 4 a tile of 64 and the
-// near words.
-// Other frames take the scattered form.
+// a voxel's inscribed sphere stays one), a bundle of at most 105 degrees (a
+// wider one crosses voxels outside the near words at depths where windows are
+// huge), a camera, grid and range within 4096 voxels, and room for its
+// tables: 20 bytes a ray, 4 a tile of 64 and the near words.  Other frames
+// take the scattered form.
+//
+// The margin.  With u = 2^-24, C1 = |S| + n and D the longest ray, a point's
+// camera coordinates are off by at most 10 u C1 (the subtraction, the rounded
+// matrix, five multiply-adds), a ray's direction by 9 u |D| (three products
+// and two sums an axis), and the walk's crossings by 3 u |D| along the ray:
+// together under 9e-7 C, C = C1 + |D|.  m = 0.002 + 1.7e-6 C is twice that (0.003
+// at 10 m / 0.05 m, 0.03 at the limits).  A ray within 0.49 - m of a centre
+// is 0.01 + m or more inside the voxel's faces there.
 inline void gather_setup(FrameArgs &a, uint8_t *base, size_t bytes) {
     Gather &g = a.ga;
     g.on = 0;
@@ -251,13 +257,18 @@ inline void gather_setup(FrameArgs &a, uint8_t *base, size_t bytes) {
     g.near_fr = g.tile + tiles;
     g.near_tr = g.near_fr + kNearWords;
 
+    double smax = 0.0;
+    for (int k = 0; k < 3; ++k) smax = std::max(smax, std::fabs((double)a.T.t[k] / a.vs) + n[k]);
+    const double m = 0.002 + 1.7e-6 * (smax + std::sqrt((double)a.vd * a.vd + (double)a.hw * a.hw + (double)a.hh * a.hh));
+    g.m = (float)m;
+    g.sphere2 = (float)((0.49 - m) * (0.49 - m));
     const double ka = (double)a.hw / a.vd, kb = (double)a.hh / a.vd;
     g.ka = (float)ka;
     g.kb = (float)kb;
     for (int side = 0; side < 4; ++side) {
-        const double *m = M + 3 * (side >> 1), k = (side >> 1 ? kb : ka) * (side & 1 ? -1.0 : 1.0);
-        const double c[3] = {std::fabs(m[0] - k * M[6]), std::fabs(m[1] - k * M[7]), std::fabs(m[2] - k * M[8])};
-        const double margin = kGatherMargin * (1.0 + std::fabs(k));
+        const double *row = M + 3 * (side >> 1), k = (side >> 1 ? kb : ka) * (side & 1 ? -1.0 : 1.0);
+        const double c[3] = {std::fabs(row[0] - k * M[6]), std::fabs(row[1] - k * M[7]), std::fabs(row[2] - k * M[8])};
+        const double margin = m * (1.0 + std::fabs(k));
         g.ew[side] = (float)(16.0 * c[0] + 0.5 * c[1] + 0.5 * c[2] + margin);
         g.ep[side] = (float)(4.0 * c[0] + 2.0 * c[1] + 0.5 * c[2] + margin);
         g.ev[side] = (float)(0.5 * (c[0] + c[1] + c[2]) + margin);
@@ -268,7 +279,7 @@ inline void gather_setup(FrameArgs &a, uint8_t *base, size_t bytes) {
     g.zv = (float)(0.5 * (std::fabs(M[6]) + std::fabs(M[7]) + std::fabs(M[8])));
     // |a - fa| <= vd (reach + margin) / (c2 - zv - margin) + margin, as in window_of
     const double reach = std::max(std::max(g.ev[0], g.ev[1]), std::max(g.ev[2], g.ev[3]));
-    g.zr = (float)(a.vd * reach / (kLateReach - 0.5 - 2.0 * kGatherMargin) + g.zv + 2.0 * kGatherMargin);
+    g.zr = (float)(a.vd * reach / (kLateReach - 0.5 - 2.0 * m) + g.zv + 2.0 * m);
     g.on = 1;
 }
 

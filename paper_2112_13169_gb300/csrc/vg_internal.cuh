@@ -102,7 +102,6 @@ struct WordBox {
 // rotation, the widths of a word's and a voxel's projection that its culling
 // compares with, and where its per-frame tables live (in the grid's loc_alt,
 // which holds nothing between calls).
-constexpr float kGatherMargin = 0.03f;   // voxels: bounds the rounding of the bundle coordinates (gather_setup)
 constexpr int kNearReach = 7;            // voxels around the camera's that the rays mark themselves
 constexpr int kLateReach = 3;            // rays around each one whose latest hit is tabled
 constexpr int kNearWords = (2 * kNearReach + 1) * (2 * kNearReach + 1);
@@ -115,6 +114,8 @@ struct Gather {
     // across the sides +a, -a, +b, -b, and along the optical axis
     float ew[4], ep[4], ev[4];
     float zw, zp, zv;
+    float m;            // margin in voxels: bounds the rounding of bundle coordinates and of the walk
+    float sphere2;      // square of the distance from a voxel's centre within which a ray visits it for certain
     float zr;           // depth from which a voxel's window lies within kLateReach - 1/2 rays of its centre
     float4 *inv;        // per ray: 1/D of the walk, 0 on an inactive axis; the latest hit around it
     uint32_t *hit;      // per ray: its hit key
