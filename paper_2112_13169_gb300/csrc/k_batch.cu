@@ -9,7 +9,7 @@
 //            K3 scattered          groups of at most 256 / LPR rays (a
 //                                  frame's rays spread over its units)
 //   phase 3b K3 gathered           32 x 8 rays (their latest hits)
-//   phase 4  K4 gathered           128 plane words of the box; 256 of slabs
+//   phase 4  K4 gathered           192 plane words of the box; 256 of slabs
 //            K4 merge              512 plane words (256 if tuned)
 // with a grid-wide barrier between phases (3b only if a frame is gathered).
 // Every frame that the gathered form can take (vg_gather.cuh) takes it here:
@@ -21,8 +21,16 @@
 // CTA finds the frame of its first unit of a phase by binary search, steps
 // forward through the frames as its units advance (see run_begin), and runs
 // the same device code as the one-step kernels (vg_units.cuh, vg_rt.cuh).
-// Reads of data an earlier phase wrote skip the L1 (LoadL2), except the ray
-// trace's occupancy loads (see group_lpr).
+// The merge's reads of data an earlier phase wrote skip the L1 (LoadL2);
+// for the inflation's and the rays' loads see there (and group_lpr).
+//
+// With 32 warps to an SM the phases are bound by latency more than by issue
+// (313 M warp instructions in 529 us, 54 % of the issue slots, for 64
+// robots), so loads run ahead (the next unit's depths in phase 1, the next
+// tile in phase 2) and the gathered units, whose cost differs most, are
+// handed out as CTAs come free: phase 1 97 -> 88 us, phase 2 60 -> 55, and
+// four steps with a read of every grid 2413 -> 2257 us (in turn: 2351); 192
+// words a phase-4 unit instead of 128 gave 2138.
 //
 // The barrier waits with a deadline (BatchCtl::bar_ns, four seconds unless
 // tuned): if the other CTAs do not all arrive in time, the waiting CTA sets
@@ -32,16 +40,20 @@
 #include "vg_rt.cuh"
 #include "vg_sync.cuh"
 
+#include <type_traits>
+
 namespace vg {
 namespace {
 
 using namespace rt;
 
-// loads of an inflate tile's staging issued together (fewer than the
-// one-step kernel's 8: this kernel's registers are capped at 64)
-constexpr int kInflateUnroll = 2;
-constexpr int kDynWords = kRtBuf * kThreads;   // also covers an inflate tile of radius <= 3
-static_assert(units::inflate_smem_words<3, 8, 8, 8>(3) <= (size_t)kDynWords, "inflate tile fits");
+// the scattered rays' buffers need kRtBuf columns, a gathered unit's lists a
+// little more; four CTAs of this fit an SM
+constexpr int kDynWords = 40 * kThreads;
+static_assert(kDynWords >= kRtBuf * kThreads, "ray buffers fit");
+// an inflate tile's staged words, twice, and its x pass
+constexpr int kStageWords = 14 * 14 * 10;
+static_assert(2 * kStageWords + 14 * 14 * 8 <= kDynWords, "inflate tiles of radius <= 3 fit");
 constexpr int kGatherWords = kBatchGatherWords;
 static_assert(sizeof(gather::GatherSmem<kGatherWords>) <= kDynWords * 4, "gathered words fit");
 static_assert(sizeof(gather::SkinSmem) <= kDynWords * 4 && sizeof(gather::LateSmem) <= kDynWords * 4 &&
@@ -80,7 +92,8 @@ __device__ __forceinline__ int64_t weighted_unit(const BatchItem *items, int n, 
 // restages that frame's arguments) only a few times.  Their units cost about
 // the same in every frame.  The inflate and merge units cost more in some
 // frames than in others (tile width and radius; how much of a grid the
-// measurement marks), so there the units go round the CTAs in turn.
+// measurement marks), so there the units go round the CTAs in turn, or, in
+// the gathered phases, as CTAs come free.
 __device__ __forceinline__ int64_t run_begin(int64_t total, unsigned b, unsigned nb) { return total * b / nb; }
 
 // The frame of unit u, given the frame i of an earlier unit of the same CTA
@@ -103,14 +116,41 @@ __device__ __forceinline__ unsigned group_lpr(const FrameArgs &a, int buffered, 
     return rt_group<LPR, units::LoadPlain>(a, S, b, grp, G, buffered, box_fr, box_tr, occ_box, buf);
 }
 
-// One inflate tile of TXW words x 8 rows x TZ slices of a batch frame.
-template <int TXW, int TZ>
-__device__ __forceinline__ void inflate_unit(const BatchItem &it, int tx, int ty, int tz, uint32_t *sm) {
+// The tile of the inflate phase's unit u, in frame i.
+struct Tile {
+    int x, y, z;
+};
+__device__ __forceinline__ Tile tile_of(const BatchItem &it, int64_t u) {
+    // a frame has fewer than 2^27 plane words, so fewer tiles
+    const uint32_t local = (uint32_t)(u - it.off[1]), t0 = (uint32_t)it.tiles[0];
+    const uint32_t t01 = local / t0;
+    return Tile{it.tile0[0] + (int)(local - t01 * t0), it.tile0[1] + (int)(t01 % (uint32_t)it.tiles[1]),
+                it.tile0[2] + (int)(t01 / (uint32_t)it.tiles[1])};
+}
+
+// One inflate tile of TXW words x 8 rows x TZ slices of a batch frame:
+// starts its staging in st, or (DO) runs its passes from there.
+template <bool DO, int TXW, int TZ>
+__device__ __forceinline__ void inflate_part(const BatchItem &it, const Tile &t, uint32_t *st, uint32_t *buf1) {
     const PlaneGeom &g = it.a.g;
+    auto part = [&](auto radius) {
+        constexpr int R = decltype(radius)::value;
+        if (DO) units::inflate_passes<R, TXW, 8, TZ>(g, it.a.pl.occ_inf, R, t.x, t.y, t.z, st, TXW + 2, 0, buf1);
+        else units::inflate_stage<R, TXW, 8, TZ>(g, it.a.pl.occ_raw, t.x, t.y, t.z, st);
+    };
     switch (it.a.r) {
-    case 1: units::inflate_tile<1, TXW, 8, TZ, units::LoadL2, kInflateUnroll>(g, it.a.pl.occ_raw, it.a.pl.occ_inf, 1, tx, ty, tz, sm); break;
-    case 2: units::inflate_tile<2, TXW, 8, TZ, units::LoadL2, kInflateUnroll>(g, it.a.pl.occ_raw, it.a.pl.occ_inf, 2, tx, ty, tz, sm); break;
-    default: units::inflate_tile<3, TXW, 8, TZ, units::LoadL2, kInflateUnroll>(g, it.a.pl.occ_raw, it.a.pl.occ_inf, 3, tx, ty, tz, sm); break;
+    case 1: part(std::integral_constant<int, 1>()); break;
+    case 2: part(std::integral_constant<int, 2>()); break;
+    default: part(std::integral_constant<int, 3>()); break;
+    }
+}
+template <bool DO>
+__device__ __forceinline__ void inflate_unit(const BatchItem &it, const Tile &t, uint32_t *st, uint32_t *buf1) {
+    switch (it.txw * 10 + it.tz) {
+    case 88: inflate_part<DO, 8, 8>(it, t, st, buf1); break;
+    case 84: inflate_part<DO, 8, 4>(it, t, st, buf1); break;
+    case 48: inflate_part<DO, 4, 8>(it, t, st, buf1); break;
+    default: inflate_part<DO, 4, 4>(it, t, st, buf1); break;
     }
 }
 
@@ -140,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
         int cur = -1;
         const int64_t lo = run_begin(ctl->total[0], blockIdx.x, nb), hi = run_begin(ctl->total[0], blockIdx.x + 1, nb);
         int i = find_item(items, n, 0, lo);
-        for (int64_t u = lo; u < hi; ++u) {
+        for (int64_t u = lo; u < hi;) {
             i = next_item(items, n, 0, u, i);   // the same for every thread
             if (i != cur) {
                 __syncthreads();   // the previous frame's copy is no longer read
@@ -153,58 +193,87 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
             const int64_t t = local * kThreads + threadIdx.x;
             if (local >= pix) {
                 gather::table_thread(s_a, t - pix * kThreads);
+                ++u;
                 continue;
             }
+            // the frame's units of this run, each one's depths loaded while
+            // the one before is placed
+            const int run = (int)(hi - u < pix - local ? hi - u : pix - local);
             switch (s_kind) {
-            case 0: units::voxelize_depth_thread<0, false, false>(s_a, t); break;
-            case 1: units::voxelize_depth_thread<0, true, false>(s_a, t); break;
-            case 2: units::voxelize_depth_thread<1, false, false>(s_a, t); break;
-            default: units::voxelize_depth_thread<1, true, false>(s_a, t); break;
+            case 0: units::voxelize_depth_run<0, false>(s_a, t, run); break;
+            case 1: units::voxelize_depth_run<0, true>(s_a, t, run); break;
+            case 2: units::voxelize_depth_run<1, false>(s_a, t, run); break;
+            default: units::voxelize_depth_run<1, true>(s_a, t, run); break;
             }
+            u += run;
         }
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->next = 0u;   // phase 3 counts from 0
     }
     if (!grid_sync(ctl, nb)) return;
 
     // ---- phase 2: inflate -------------------------------------------------
     {
         // units in turn over the CTAs: their cost differs between frames,
-        // and interleaving keeps the CTAs' shares even
+        // and interleaving keeps the CTAs' shares even.  A tile is staged
+        // while the one before it is worked on.  (No SM reads occ_raw in this
+        // launch before this phase, so its L1 holds no older state of it.)
+        const int64_t total = ctl->total[1];
         int i = find_item(items, n, 1, blockIdx.x);
-        for (int64_t u = blockIdx.x; u < ctl->total[1]; u += nb) {
-            i = next_item(items, n, 1, u, i);
-            const BatchItem &it = items[i];
-            // a frame has fewer than 2^27 plane words, so fewer tiles
-            const uint32_t local = (uint32_t)(u - it.off[1]), t0 = (uint32_t)it.tiles[0];
-            const uint32_t t01 = local / t0;
-            const int tx = it.tile0[0] + (int)(local - t01 * t0);
-            const int ty = it.tile0[1] + (int)(t01 % (uint32_t)it.tiles[1]);
-            const int tz = it.tile0[2] + (int)(t01 / (uint32_t)it.tiles[1]);
-            switch (it.txw * 10 + it.tz) {
-            case 88: inflate_unit<8, 8>(it, tx, ty, tz, dyn); break;
-            case 84: inflate_unit<8, 4>(it, tx, ty, tz, dyn); break;
-            case 48: inflate_unit<4, 8>(it, tx, ty, tz, dyn); break;
-            default: inflate_unit<4, 4>(it, tx, ty, tz, dyn); break;
+        Tile t = {};
+        if (blockIdx.x < total) {
+            t = tile_of(items[i], blockIdx.x);
+            inflate_unit<false>(items[i], t, dyn, nullptr);
+        }
+        uint32_t *st = dyn, *other = dyn + kStageWords;
+        for (int64_t u = blockIdx.x; u < total; u += nb) {
+            int j = i;
+            Tile tj = {};
+            if (u + nb < total) {
+                j = next_item(items, n, 1, u + nb, i);
+                tj = tile_of(items[j], u + nb);
+                inflate_unit<false>(items[j], tj, other, nullptr);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
             }
+            __syncthreads();
+            inflate_unit<true>(items[i], t, st, dyn + 2 * kStageWords);   // ends with a barrier
+            i = j;
+            t = tj;
+            uint32_t *const swap = st;
+            st = other;
+            other = swap;
         }
     }
     if (!grid_sync(ctl, nb)) return;
 
     // ---- phase 3, gathered: around the camera, and the skin ---------------
-    // units in turn over the CTAs: their cost differs between and within
-    // frames.  (Here and in the phases after it frame i's arguments are
+    // units go to the CTAs as these come free: their cost differs between
+    // and within frames.  (Here and in the phases after it frame i's arguments are
     // staged for every unit: a CTA's units lie far apart.)
     auto stage = [&](int i) {
         __syncthreads();   // the previous copy is no longer read
         stage_args(items[i].a, s_a);
         __syncthreads();
     };
+    // The next unit of this CTA: its first is its own, the others are handed
+    // out.  Thread 0 asks as the unit before begins.
+    __shared__ uint32_t s_next;
+    auto ask = [&]() { return threadIdx.x == 0 ? nb + atomicAdd(&ctl->next, 1u) : 0u; };
+    auto told = [&](uint32_t asked) {
+        if (threadIdx.x == 0) s_next = asked;
+        __syncthreads();
+        return (int64_t)s_next;
+    };
     {
         float S[3];
         int32_t v0[3];
-        int i = 0;
-        for (int64_t u = blockIdx.x; u < ctl->total[4]; u += nb) {
-            i = u == blockIdx.x ? find_item(items, n, 4, u) : next_item(items, n, 4, u, i);
+        uint32_t asked = 0;
+        int i = blockIdx.x < ctl->total[4] ? find_item(items, n, 4, blockIdx.x) : 0;
+        for (int64_t u = blockIdx.x; u < ctl->total[4]; u = told(asked)) {
+            i = next_item(items, n, 4, u, i);
             stage(i);
+            asked = ask();
             gather::frame_start(s_a, S, v0);
             const int32_t local = (int32_t)(u - __ldg(&items[i].off[4])), near = __ldg(&items[i].near_units);
             if (local < near)
@@ -263,6 +332,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
     // ---- phase 3b: the latest hits of the gathered frames' rays -----------
     if (ctl->total[5]) {
         int i = 0;
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->next = 0u;   // and phase 4
         for (int64_t u = blockIdx.x; u < ctl->total[5]; u += nb) {
             i = u == blockIdx.x ? find_item(items, n, 5, u) : next_item(items, n, 5, u, i);
             stage(i);
@@ -274,15 +344,16 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
 
     // ---- phase 4: merge ---------------------------------------------------
     {
-        // units in turn over the CTAs: their cost differs between frames,
-        // and interleaving keeps the CTAs' shares even
         float S[3];
         int32_t v0[3];
+        const bool handed = ctl->total[5] != 0;   // (a batch of scattered frames alone: in turn)
+        uint32_t asked = 0;
         int i = find_item(items, n, 3, blockIdx.x);
-        for (int64_t u = blockIdx.x; u < ctl->total[3]; u += nb) {
+        for (int64_t u = blockIdx.x; u < ctl->total[3]; u = handed ? told(asked) : u + nb) {
             i = next_item(items, n, 3, u, i);
             const BatchItem &it = items[i];
             const int64_t local = u - __ldg(&it.off[3]);
+            if (handed) asked = ask();
             if (__ldg(&it.a.ga.on)) {
                 stage(i);
                 const int32_t box = __ldg(&it.box_units);
@@ -298,6 +369,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
             // the unit's mwpu plane words, one or two per thread
             for (int k = 0; k < it.mwpu; k += kThreads)
                 units::merge_word<units::LoadL2>(it.a.g, it.a.pl, it.a.loc, it.a.ring, local * it.mwpu + k + threadIdx.x);
+            if (handed) __syncthreads();   // s_next is no longer read
         }
     }
 }

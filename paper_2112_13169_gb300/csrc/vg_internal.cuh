@@ -181,13 +181,16 @@ struct BatchItem {
 // pending re-centre, unless tuned (other frames' units are 256 words, one
 // per thread).
 constexpr int kBatchMergeWords = 512;
-// Plane words per phase-4 unit of a gathered frame of a batch.
-constexpr int kBatchGatherWords = 128;
+// Plane words per phase-4 unit of a gathered frame of a batch.  A unit's
+// staging and its chain of phases cost about 7 us however few its words, and
+// its lists' shared memory comes out of the L1 (64 words: 2626 us for four
+// steps of 64 robots; 128: 2257, 160: 2173, 192: 2138, 256: 2250).
+constexpr int kBatchGatherWords = 192;
 
 // Control block of a batch launch, copied to the device with the items.
 struct BatchCtl {
     int32_t n;          // frames
-    int32_t pad0;
+    uint32_t next;      // phases 3 and 4, gathered: units handed out beyond one per CTA (the kernel zeroes it)
     int64_t total[6];   // units per phase, as BatchItem::off
     unsigned bar_count; // grid barrier: arrivals
     unsigned bar_gen;   // grid barrier: generation

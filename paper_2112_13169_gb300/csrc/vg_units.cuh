@@ -145,14 +145,12 @@ __device__ __forceinline__ void count_points(const FrameArgs &a, unsigned kept) 
     if ((threadIdx.x & 31) == 0 && total) atomicAdd(a.stats + 1, (unsigned long long)total);
 }
 
-// Pixels 4t .. 4t+3 of the image.  DT: 0 = f32, 1 = u16.  VEC: the image
-// base is aligned for a 4-pixel load.  Warp-synchronous: every lane of the
-// warp must call this (threads past the image do nothing).
-template <int DT, bool VEC, bool SCAN = true>
-__device__ __forceinline__ void voxelize_depth_thread(const FrameArgs &a, int64_t t) {
+// The depths of pixels 4t .. 4t+3 of the image (0 past its end).  DT: 0 =
+// f32, 1 = u16.  VEC: the image base is aligned for a 4-pixel load.
+template <int DT, bool VEC>
+__device__ __forceinline__ void load_depths(const FrameArgs &a, int64_t t, float d[4]) {
     const int64_t npix = (int64_t)a.W * a.H;
     const int64_t p0 = t * 4;
-    float d[4];
     if (VEC && p0 + 3 < npix) {
         if (DT == 0) {
             const float4 q = __ldg(reinterpret_cast<const float4 *>(a.depth) + (p0 >> 2));
@@ -174,6 +172,14 @@ __device__ __forceinline__ void voxelize_depth_thread(const FrameArgs &a, int64_
             }
         }
     }
+}
+
+// Pixels 4t .. 4t+3 of the image, of depths d.  Warp-synchronous: every lane
+// of the warp must call this (threads past the image do nothing).
+template <bool SCAN>
+__device__ __forceinline__ void voxelize_depths(const FrameArgs &a, int64_t t, const float d[4]) {
+    const int64_t npix = (int64_t)a.W * a.H;
+    const int64_t p0 = t * 4;
     uint32_t key[4], bit[4];
     // images hold fewer than 2^31 pixels, so p0 (at most 1023 past the last
     // one) fits 32 bits
@@ -200,6 +206,27 @@ __device__ __forceinline__ void voxelize_depth_thread(const FrameArgs &a, int64_
 #pragma unroll
     for (int j = 0; j < 4; ++j) warp_set_bits<SCAN>(a.pl.occ_raw, key[j], bit[j]);
     count_points(a, kept);
+}
+
+template <int DT, bool VEC>
+__device__ __forceinline__ void voxelize_depth_thread(const FrameArgs &a, int64_t t) {
+    float d[4];
+    load_depths<DT, VEC>(a, t, d);
+    voxelize_depths<true>(a, t, d);
+}
+
+// The same for `units` threads 256 apart, from t on, each one's depths loaded
+// while the one before is placed.
+template <int DT, bool VEC>
+__device__ __forceinline__ void voxelize_depth_run(const FrameArgs &a, int64_t t, int units) {
+    float d[4], next[4];
+    load_depths<DT, VEC>(a, t, next);
+    for (int k = 0; k < units; ++k, t += 256) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) d[j] = next[j];
+        if (k + 1 < units) load_depths<DT, VEC>(a, t + 256, next);
+        voxelize_depths<false>(a, t, d);
+    }
 }
 
 // The word and bit of point i of the cloud (kNoWord past its end).
@@ -363,6 +390,27 @@ __device__ __forceinline__ void inflate_tile(const PlaneGeom &g, const uint32_t 
     }
     __syncthreads();
     inflate_passes<R, TXW, TY, TZ>(g, out, r_rt, tile_x, tile_y, tile_z, buf0, hx, 0, buf1);
+}
+
+// Starts the copies that stage a tile of radius R (zeros outside the grid):
+// one commit group of this thread's, to be waited for.  They may go through
+// the L1, so nothing on this SM may have read an older state of the plane in
+// this launch.  CTA-cooperative.
+template <int R, int TXW, int TY, int TZ>
+__device__ __forceinline__ void inflate_stage(const PlaneGeom &g, const uint32_t *raw, int tile_x, int tile_y, int tile_z,
+                                              uint32_t *st) {
+    constexpr int hx = TXW + 2, hy = TY + 2 * R, hz = TZ + 2 * R;
+    const int w0 = tile_x * TXW, y0 = tile_y * TY, z0 = tile_z * TZ;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(st);
+    for (int i = threadIdx.x; i < hz * hy * hx; i += 256) {
+        const int lx = i % hx, rest = i / hx, ly = rest % hy, lz = rest / hy;
+        const int w = w0 + lx - 1, y = y0 + ly - R, z = z0 + lz - R;
+        const bool in = (unsigned)w < (unsigned)g.wx && (unsigned)y < (unsigned)g.ny && (unsigned)z < (unsigned)g.nz;
+        const uint32_t *src = in ? raw + ((int64_t)z * g.ny + y) * g.wx + w : raw;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 4u * i), "l"(src), "r"(in ? 4 : 0)
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------

@@ -12,7 +12,7 @@ import numpy as np
 import pytest
 
 from gridcheck import assert_grid, oracle_grid
-from synth import make
+from synth import body_pose, make
 
 pytestmark = pytest.mark.gpu
 
@@ -269,3 +269,52 @@ def test_batch_rejects_bad_frames(vg):
     batch.close()
     big.close()
     g.close()
+
+
+# grid, voxel, field of view (past 105 degrees a frame keeps the scattered
+# form), radius, image (odd: pixels past the last whole four, rows not aligned)
+BOTH = [((33, 9, 5), 0.2, 80, 1, (61, 47)), ((129, 70, 33), 0.1, 120, 3, (160, 121)),
+        ((260, 37, 18), 0.1, 90, 2, (99, 64)), ((40, 41, 42), 0.1, 120, 1, (1, 1)),
+        ((300, 130, 70), 0.05, 85, 3, (321, 240)), ((64, 64, 64), 0.1, 60, 2, (7, 3))]
+
+
+@pytest.mark.parametrize("copies", [1, 12])
+def test_batch_of_both_forms_at_odd_sizes(vg, copies):
+    """Gathered and scattered frames in one batch, from fewer units a phase
+    than CTAs to several rounds, and a frame's pixels from an odd address."""
+    from oracle import OracleGrid, OracleParams
+    rng = np.random.default_rng(7)
+    grids, oracles, frames = [], [], []
+    for c in range(copies):
+        for k, (n, vs, fov, r, (w, h)) in enumerate(BOTH):
+            depth = float(np.float32(0.45 * max(n) * vs))
+            pos = (0.3 * c, -0.2 * k, 0.1)
+            grids.append(vg.Grid(n, vs, fov, fov - 20, depth, r, pos))
+            oracles.append(OracleGrid(OracleParams(n, vs, fov, fov - 20, depth, r), pos))
+            d = rng.uniform(0.3, 1.1, (h, w)).astype(np.float32) * np.float32(depth)
+            if k % 2:
+                img = np.rint(d * 1000).astype(np.uint16)
+                scale = 1e-3
+            else:
+                img, scale = d, 1.0
+            base = torch.zeros(img.size + 1, dtype=torch.uint16 if k % 2 else torch.float32, device="cuda")
+            base[1:] = torch.from_numpy(img.reshape(-1)).cuda()
+            T = body_pose(np.array(pos) + 0.03, 0.5 * c + k)
+            frames.append((img, base[1:].view(h, w), T, scale))
+    batch = vg.Batch(len(grids))
+    try:
+        for step in range(2):
+            to = [tuple(0.21 * (step + 1) * np.array([1.0, -1.0, 0.5])) for o in oracles]
+            batch.step([(g, f[1], f[2], p, f[3]) for g, f, p in zip(grids, frames, to)])
+            for g, o, (img, _, T, scale), p in zip(grids, oracles, frames, to):
+                o.integrate_depth(T, img, scale)
+                o.shift(p)
+        assert batch.status() == vg.VG_OK
+        for g, o in zip(grids, oracles):
+            got, origin = _read(g)
+            assert list(origin) == list(o.o)
+            assert np.array_equal(got.reshape(o.loc.shape), o.loc)
+    finally:
+        batch.close()
+        for g in grids:
+            g.close()
