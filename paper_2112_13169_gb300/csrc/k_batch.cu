@@ -2,7 +2,7 @@
 //
 // One cooperative launch of k_batch runs, for every frame of a batch (each
 // with its own grid, resolution, voxel size and radius), the whole path:
-//   phase 1  K1 voxelize           units of 1024 pixels; 256 rays of the table
+//   phase 1  K1 voxelize           tiles of 32 x 32 pixels; 256 rays of the table
 //   phase 2  K2 inflate            8 (or 4) words x 8 rows x 8 (or 4)
 //                                  slices (radius 1..3) of the frame's box
 //   phase 3  K3 gathered           256 rays around the camera; 256 words
@@ -177,6 +177,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
 
     // ---- phase 1: voxelize ------------------------------------------------
     {
+        units::WordTab &tab = *reinterpret_cast<units::WordTab *>(dyn);
+        units::tab_clear(tab);   // (the first frame's staging ends with a barrier)
         int cur = -1;
         const int64_t lo = run_begin(ctl->total[0], blockIdx.x, nb), hi = run_begin(ctl->total[0], blockIdx.x + 1, nb);
         int i = find_item(items, n, 0, lo);
@@ -190,9 +192,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
                 cur = i;
             }
             const int64_t local = u - __ldg(&items[i].off[0]), pix = __ldg(&items[i].pix_units);
-            const int64_t t = local * kThreads + threadIdx.x;
             if (local >= pix) {
-                gather::table_thread(s_a, t - pix * kThreads);
+                gather::table_thread(s_a, (local - pix) * kThreads + threadIdx.x);
                 ++u;
                 continue;
             }
@@ -200,10 +201,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
             // the one before is placed
             const int run = (int)(hi - u < pix - local ? hi - u : pix - local);
             switch (s_kind) {
-            case 0: units::voxelize_depth_run<0, false>(s_a, t, run); break;
-            case 1: units::voxelize_depth_run<0, true>(s_a, t, run); break;
-            case 2: units::voxelize_depth_run<1, false>(s_a, t, run); break;
-            default: units::voxelize_depth_run<1, true>(s_a, t, run); break;
+            case 0: units::voxelize_run<0, false>(s_a, (int32_t)local, run, tab); break;
+            case 1: units::voxelize_run<0, true>(s_a, (int32_t)local, run, tab); break;
+            case 2: units::voxelize_run<1, false>(s_a, (int32_t)local, run, tab); break;
+            default: units::voxelize_run<1, true>(s_a, (int32_t)local, run, tab); break;
             }
             u += run;
         }

@@ -1,5 +1,5 @@
-// K1 as its own launch: one thread per four pixels (or per point); the work
-// itself is in vg_units.cuh.
+// K1 as its own launch: a CTA per tile of pixels, a thread per point; the
+// work itself is in vg_units.cuh.
 #include "vg_gather.cuh"
 
 #include <algorithm>
@@ -15,6 +15,7 @@ namespace {
 // The first `ntab` CTAs write the gathered form's ray table instead.
 template <int DT, bool VEC>
 __global__ void __launch_bounds__(256) k_voxelize_depth(const FrameArgs a, const int early, const int ntab) {
+    __shared__ units::WordTab tab;
     pdl_wait();   // the depth image and the planes belong to earlier work
     if (early) pdl_trigger();
     if ((int)blockIdx.x < ntab) {
@@ -23,7 +24,7 @@ __global__ void __launch_bounds__(256) k_voxelize_depth(const FrameArgs a, const
     }
     const unsigned block = blockIdx.x - ntab;
     if (a.rt_next && block == 0 && threadIdx.x == 0) *a.rt_next = 0u;   // K3 of this frame counts from 0
-    units::voxelize_depth_thread<DT, VEC>(a, (int64_t)block * blockDim.x + threadIdx.x);
+    units::voxelize_tile<DT, VEC>(a, (int32_t)block, tab);
 }
 
 __global__ void __launch_bounds__(256) k_voxelize_points(const FrameArgs a, const int early, const int ntab) {
@@ -85,16 +86,13 @@ constexpr int64_t kDenseBlocks = 152;   // one to an SM
 
 cudaError_t launch_voxelize_depth(const FrameArgs &a, int32_t dtype, cudaStream_t s, const Sched &sc) {
     const int early = sc.early_inflate;
-    const int64_t npix = (int64_t)a.W * a.H;
-    const int64_t threads = (npix + 3) / 4;
     const int ntab = (int)((gather::table_threads(a) + 255) / 256);
-    const unsigned blocks = (unsigned)((threads + 255) / 256) + ntab;
-    const uintptr_t base = reinterpret_cast<uintptr_t>(a.depth);
+    const unsigned blocks = (unsigned)units::pixel_tiles(a.W, a.H) + ntab;
     if (dtype == 0) {
-        if (base % 16 == 0) return launch_pdl(k_voxelize_depth<0, true>, blocks, 256, 0, s, a, early, ntab);
+        if (units::pixels_aligned(a.depth, a.W, 4)) return launch_pdl(k_voxelize_depth<0, true>, blocks, 256, 0, s, a, early, ntab);
         return launch_pdl(k_voxelize_depth<0, false>, blocks, 256, 0, s, a, early, ntab);
     }
-    if (base % 8 == 0) return launch_pdl(k_voxelize_depth<1, true>, blocks, 256, 0, s, a, early, ntab);
+    if (units::pixels_aligned(a.depth, a.W, 2)) return launch_pdl(k_voxelize_depth<1, true>, blocks, 256, 0, s, a, early, ntab);
     return launch_pdl(k_voxelize_depth<1, false>, blocks, 256, 0, s, a, early, ntab);
 }
 

@@ -90,3 +90,31 @@ def test_clouds_around_the_shared_plane_rule(vg, n, more):
     T = body_pose([0.02, 0.0, -0.01], 0.3, 0.0, 0.1)
     points = check_cloud(vg, n, 0.1, xyz, T, "%d points" % len(xyz))
     assert 0 < points < 2 * len(xyz)
+
+
+# tiles of 32 x 32 pixels: one pixel, a tile less and more a pixel, rows that
+# are and are not whole fours; a far noisy image fills a tile's table (1,024
+# words where it has 256 slots), a flat one shares a few words
+@pytest.mark.parametrize("w,h", [(1, 1), (31, 33), (32, 32), (36, 31), (68, 65), (97, 1), (1, 97)])
+@pytest.mark.parametrize("dtype", [np.float32, np.uint16])
+def test_images_around_tiles(vg, w, h, dtype):
+    n, vs = (96, 120, 120), 0.1
+    rng = np.random.default_rng(w * 100 + h)
+    for off in (0, 1):   # the image's address whole and not whole fours of pixels
+        g = vg.Grid(n, vs, 80.0, 70.0, 4.0, 0, (0.0, 0.0, 0.0), flags=vg.VG_FLAG_STATS)
+        o = OracleGrid(OracleParams(n, vs, 80.0, 70.0, 4.0, 0), (0.0, 0.0, 0.0))
+        out = torch.empty(g.nvox, dtype=torch.uint8, device="cuda")
+        for flat in (False, True):
+            d = rng.uniform(1.9 if flat else 0.4, 2.0 if flat else 5.9, (h, w))
+            d[rng.random((h, w)) < 0.05] = 0
+            d = np.rint(d * 1000).astype(dtype) if dtype == np.uint16 else d.astype(dtype)
+            scale = 1e-3 if dtype == np.uint16 else 1.0
+            buf = torch.zeros(w * h + off, dtype=torch.uint16 if dtype == np.uint16 else torch.float32, device="cuda")
+            buf[off:] = torch.from_numpy(d.reshape(-1)).cuda()
+            T = body_pose([0.0, 0.0, 0.0], rng.uniform(-3, 3), 0.2, 0.1)
+            g.integrate_depth(buf[off:].view(h, w), T, scale)
+            o.integrate_depth(T, d, scale)
+            g.read(out)
+            torch.cuda.synchronize()
+            assert_same(out.cpu().numpy().reshape(g.shape), o.loc, "%dx%d, offset %d, flat %s" % (w, h, off, flat))
+        g.close()
