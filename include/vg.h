@@ -320,6 +320,9 @@ VG_API int vg_batch_status(vg_batch *batch);
  *                             default; 0 selects it) or 4.
  *  VG_TUNE_BATCH_MERGE_WORDS  plane words per merge unit (phase 4): 512 (the
  *                             default; 0 selects it) or 256.
+ *                             (A frame whose K3 and K4 are gathered, see
+ *                             VG_TUNE_RT_LANES, takes neither this knob
+ *                             nor the lanes and the spread.)
  *  VG_TUNE_BATCH_SPREAD       how phase 3 (the ray trace) shares its units,
  *                             groups of 256 / LPR rays, among the CTAs' contiguous
  *                             runs.  1 (default): each frame's rays are
@@ -534,7 +537,7 @@ VG_API int vg_profile_read(vg_grid *grid, double ms[VG_NKERNELS], int64_t timed[
  *                    thread) or 512 (two per thread).
  *  VG_TUNE_INFLATE_TMA
  *                    1 (default): K2 moves each tile's raw words with one
- *                    tensor-memory-accelerator copy (radius 1..3); 0: its
+ *                    tensor-memory-accelerator copy (any radius); 0: its
  *                    threads load them.
  *  VG_TUNE_EARLY_INFLATE
  *                    1 (default): K2's CTAs launch while K1 runs, as soon

@@ -1,7 +1,7 @@
 // K2 as its own launch: one CTA per 8-word x 8-row x 8-slice tile of the
-// occupancy plane (4 slices for grids of one to four such tiles per SM);
-// the work itself is in vg_units.cuh.  For r = 1, 2, 3 the
-// radius is a compile-time constant; other radii use a runtime radius.
+// frame's box (4 slices for one to four such tiles per SM); the work itself
+// is in vg_units.cuh.  For r = 1, 2, 3 the radius is a compile-time constant;
+// other radii use a runtime radius.
 #include "vg_units.cuh"
 
 #include <cuda.h>

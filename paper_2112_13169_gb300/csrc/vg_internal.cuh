@@ -221,7 +221,7 @@ struct Sched {
     int32_t inflate_tile = kTileAuto;
     int32_t rt_ctas = 0;        // K3 CTAs per SM; 0: as many as fit
     int32_t merge_words = 256;  // plane words per CTA of K4: 256 (one per thread) or 512 (two)
-    int32_t inflate_tma = 1;    // K2 stages its tiles with tensor-memory-accelerator copies (radius 1..3)
+    int32_t inflate_tma = 1;    // K2 stages its tiles with tensor-memory-accelerator copies
     int32_t early_inflate = 1;  // K2 launches while K1 runs (else when K1 completes)
 };
 
