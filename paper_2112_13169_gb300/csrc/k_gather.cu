@@ -64,7 +64,9 @@ cudaError_t launch_rayhit(const FrameArgs &a, cudaStream_t s) {
 // each, one phase after another, so a CTA of few words ends sooner and one of
 // many spends less on its barriers and rounds.  Measured (a frame with its
 // read, CTAs of 64 / 128 / 256 words): a box of 40 k words 35 / 38 / 52 us, of
-// 76 k 44 / 41 / 47, of 200 k 83 / 77 / 77, of 600 k 203 / 174 / 163.
+// 76 k 44 / 41 / 47, of 200 k 83 / 77 / 77, of 600 k 203 / 174 / 163.  CTAs of
+// 128 threads, whose barriers hold fewer warps, and of 512 lose as well:
+// three 640x480 frames with their read 157 to 189 and 170 us against 148.
 cudaError_t launch_gather(const FrameArgs &a, cudaStream_t s) {
     const int64_t words = (int64_t)a.box.nw * a.box.ny * a.box.nz;
     if (words < 45000) return gather_words<64>(a, s);
