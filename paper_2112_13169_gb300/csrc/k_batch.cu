@@ -12,9 +12,10 @@
 //   phase 4  K4 gathered           192 plane words of the box; 256 of slabs
 //            K4 merge              512 plane words (256 if tuned)
 // with a grid-wide barrier between phases (3b only if a frame is gathered).
-// Every frame that the gathered form can take (vg_gather.cuh) takes it here:
-// many frames fill the device, so its fewer instructions count and the
-// latency of its phases does not (the one-frame launch has a rule on sizes).  A frame's re-centre (K5) is not
+// A batch whose frames that the gathered form can take (vg_gather.cuh) hold
+// enough voxels together (kBatchGatherVoxels) has them gathered: many frames
+// fill the device, so its fewer instructions count and the latency of its
+// phases does not.  A frame's re-centre (K5) is not
 // a phase: it moves its grid's ring, and that grid's next merge sets the
 // voxels it brought in to unknown (Ring).
 // Units of every frame are laid end to end per phase (BatchItem::off).  A

@@ -918,6 +918,7 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
     vg::BatchCtl *ctl = reinterpret_cast<vg::BatchCtl *>(B->host);
     vg::BatchItem *items = reinterpret_cast<vg::BatchItem *>(B->host + sizeof(vg::BatchCtl));
     int64_t total[6] = {0, 0, 0, 0, 0, 0};
+    double voxels = 0.0;   // of the frames that could be gathered
     for (int32_t i = 0; i < n; ++i) {
         const vg_frame &f = frames[i];
         vg_grid *G = f.grid;
@@ -927,6 +928,14 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
         std::memset(&it, 0, sizeof(it));
         it.a = depth_frame_args(G, T, f.depth, f.width, f.height, f.dtype, f.depth_scale);
         if (G->p.flags == 0) vg::host::gather_setup(it.a, G->loc_alt, (size_t)G->g.nvox + 16);
+        if (it.a.ga.on) voxels += vg::host::gather_voxels(it.a);
+    }
+    const bool gather = voxels >= vg::host::kBatchGatherVoxels;
+    for (int32_t i = 0; i < n; ++i) {
+        const vg_frame &f = frames[i];
+        vg_grid *G = f.grid;
+        vg::BatchItem &it = items[i];
+        it.a.ga.on = it.a.ga.on && gather;
         // the merge writes through the grid's ring and sets what a pending
         // re-centre brought in to unknown
         it.a.ring = ring_of(G);

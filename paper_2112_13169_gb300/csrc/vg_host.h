@@ -203,11 +203,21 @@ inline void depth_box(FrameArgs &a, const vg_params *p, double tx, double ty) {
 // of 43 voxels: 28 against 22 us), above it is (21,201 of 100: 41.4 against
 // 45.3; 33,221 of 125: 56 against 70; 132,525 of 250: 163 against 350).
 constexpr double kGatherVoxels = 250e3;
-inline bool gather_pays(const FrameArgs &a) {
+inline double gather_voxels(const FrameArgs &a) {
     const double rays = (2.0 * a.hw + 1.0) * (2.0 * a.hh + 1.0);
     const double box = 32.0 * a.box.nw * a.box.ny * a.box.nz;
-    return std::min(rays * a.vd / 3.0, box / 2.0) >= kGatherVoxels;
+    return std::min(rays * a.vd / 3.0, box / 2.0);
 }
+inline bool gather_pays(const FrameArgs &a) { return gather_voxels(a) >= kGatherVoxels; }
+
+// A batch's frames are gathered together or not at all (one gathered frame
+// brings the launch a phase and a barrier more): from kBatchGatherVoxels in
+// all, by the same count.  Measured, a step gathered against scattered: 4
+// frames of 320x240 into 80 x 80 x 40 (185 k) 63 against 49 us, 8 (370 k) 70
+// against 62, 12 (554 k) 68 against 70; into 100 x 100 x 20, 2 (200 k) 59
+// against 48, 4 (400 k) 60 against 60, 8 (800 k) 65 against 75, 16 84 against
+// 106; one 640x480 frame into 200 x 200 x 100 (707 k) 63 against 71.
+constexpr double kBatchGatherVoxels = 450e3;
 
 // Sets up the gathered form of a frame (vg_gather.cuh) in `bytes` bytes of
 // device memory at base (256-byte aligned), or leaves it off: a.T, a.vs, the
