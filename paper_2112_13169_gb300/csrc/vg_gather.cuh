@@ -52,6 +52,7 @@
 #pragma once
 
 #include "vg_units.cuh"
+#include "vg_window.cuh"
 
 #include <type_traits>
 
@@ -59,7 +60,6 @@ namespace vg {
 namespace gather {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kThreads = 256;
 constexpr uint32_t kNoHit = 0xffffffffu;
 constexpr uint32_t kNone = 0xfffffffeu;   // no ray's key: no ray has a certain say
 constexpr int kNear = kNearReach, kNearN = 2 * kNear + 1, kNearRows = kNearWords;
@@ -138,106 +138,11 @@ __device__ __forceinline__ bool visits(const float4 &r, const float S[3], const 
     return ok && in < out && in < (0x3f800000u << 2);   // t < 1
 }
 
-// A point in camera axes, voxels from the camera.
-struct Place {
-    float c0, c1, c2;
-};
-
-__device__ __forceinline__ Place place_of(const Gather &g, float rx, float ry, float rz) {
-    Place p;
-    p.c0 = __fmaf_rn(g.M[2], rz, __fmaf_rn(g.M[1], ry, g.M[0] * rx));
-    p.c1 = __fmaf_rn(g.M[5], rz, __fmaf_rn(g.M[4], ry, g.M[3] * rx));
-    p.c2 = __fmaf_rn(g.M[8], rz, __fmaf_rn(g.M[7], ry, g.M[6] * rx));
-    return p;
-}
-
-// Whether a box around p with reaches e (sides +a, -a, +b, -b) and z may
-// touch the bundle.
-__device__ __forceinline__ bool in_bundle(const FrameArgs &a, const Place &p, const float e[4], float z) {
-    const Gather &g = a.ga;
-    return __fmaf_rn(-g.ka, p.c2, p.c0) <= e[0] && __fmaf_rn(-g.ka, p.c2, -p.c0) <= e[1] &&
-           __fmaf_rn(-g.kb, p.c2, p.c1) <= e[2] && __fmaf_rn(-g.kb, p.c2, -p.c1) <= e[3] &&
-           p.c2 + z + g.m >= 0.0f && p.c2 - z - g.m <= (float)a.vd;
-}
-
-struct Window {
-    int32_t alo, ahi, blo, bhi;   // rays a in [alo, ahi], b in [blo, bhi]; empty if lo > hi
-    uint32_t kmin;                // no ray enters the box with a key of kmin or less
-    __device__ __forceinline__ int32_t count() const { return max(ahi - alo + 1, 0) * max(bhi - blo + 1, 0); }
-};
-
-// The window of a box with half sizes (hx, 1/2, 1/2) around p, z its reach
-// along the optical axis: |a - fa| <= vd (its reach across the plane through
-// the camera and its centre) / (its nearest depth).
-__device__ __forceinline__ Window window_of(const FrameArgs &a, const Place &p, float hx, float z) {
-    const Gather &g = a.ga;
-    const float fvd = (float)a.vd, fw = (float)a.hw, fh = (float)a.hh;
-    Window w;
-    const float zn = p.c2 - z - g.m;
-    w.kmin = __float_as_uint(fminf(fmaxf(__fdividef(zn, fvd), 0.0f), 1.0f)) << 2;
-    if (zn < 0.2f) {
-        w.alo = -a.hw; w.ahi = a.hw; w.blo = -a.hh; w.bhi = a.hh;
-        return w;
-    }
-    const float iz = __fdividef(1.0f, p.c2), k0 = p.c0 * iz, k1 = p.c1 * iz, q = __fdividef(fvd, zn);
-    const float h0 = hx * fabsf(__fmaf_rn(-k0, g.M[6], g.M[0])) +
-                     0.5f * (fabsf(__fmaf_rn(-k0, g.M[7], g.M[1])) + fabsf(__fmaf_rn(-k0, g.M[8], g.M[2])));
-    const float h1 = hx * fabsf(__fmaf_rn(-k1, g.M[6], g.M[3])) +
-                     0.5f * (fabsf(__fmaf_rn(-k1, g.M[7], g.M[4])) + fabsf(__fmaf_rn(-k1, g.M[8], g.M[5])));
-    const float wa = __fmaf_rn(h0 + g.m, q, g.m), wb = __fmaf_rn(h1 + g.m, q, g.m);
-    const float fa = k0 * fvd, fb = k1 * fvd;
-    w.alo = (int32_t)ceilf(fmaxf(fa - wa, -fw));
-    w.ahi = (int32_t)floorf(fminf(fa + wa, fw));
-    w.blo = (int32_t)ceilf(fmaxf(fb - wb, -fh));
-    w.bhi = (int32_t)floorf(fminf(fb + wb, fh));
-    return w;
-}
-
-// The window of the face of voxel i that a walk enters through along axis k:
-// the projections of its corners, the margin beyond its edges.
-__device__ __forceinline__ Window face_window(const FrameArgs &a, const float S[3], const int32_t v0[3],
-                                              const int32_t i[3], int k) {
-    const Gather &g = a.ga;
-    const float fvd = (float)a.vd, fw = (float)a.hw, fh = (float)a.hh;
-    const float span = 1.0f + 2.0f * g.m;
-    float r[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-        r[j] = (j == k ? (float)(i[j] + (i[j] < v0[j])) : (float)i[j] - g.m) - S[j];
-    const Place p = place_of(g, r[0], r[1], r[2]);
-    const int k1 = k == 0 ? 1 : 0, k2 = k == 2 ? 1 : 2;
-    const float u0 = span * g.M[k1], u1 = span * g.M[3 + k1], u2 = span * g.M[6 + k1];
-    const float w0 = span * g.M[k2], w1 = span * g.M[3 + k2], w2 = span * g.M[6 + k2];
-    Window w;
-    const float zn = p.c2 + fminf(u2, 0.0f) + fminf(w2, 0.0f) - g.m;
-    w.kmin = __float_as_uint(fminf(fmaxf(__fdividef(zn, fvd), 0.0f), 1.0f)) << 2;
-    if (zn < 0.2f) {
-        w.alo = -a.hw; w.ahi = a.hw; w.blo = -a.hh; w.bhi = a.hh;
-        return w;
-    }
-    float alo = INFINITY, ahi = -INFINITY, blo = INFINITY, bhi = -INFINITY;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const float x = p.c0 + (c & 1 ? u0 : 0.0f) + (c & 2 ? w0 : 0.0f), y = p.c1 + (c & 1 ? u1 : 0.0f) + (c & 2 ? w1 : 0.0f);
-        const float q = __fdividef(fvd, p.c2 + (c & 1 ? u2 : 0.0f) + (c & 2 ? w2 : 0.0f));
-        alo = fminf(alo, x * q);
-        ahi = fmaxf(ahi, x * q);
-        blo = fminf(blo, y * q);
-        bhi = fmaxf(bhi, y * q);
-    }
-    const float m = __fmaf_rn(2.5f * g.m, __fdividef(fvd, zn), g.m);
-    w.alo = (int32_t)ceilf(fmaxf(alo - m, -fw));
-    w.ahi = (int32_t)floorf(fminf(ahi + m, fw));
-    w.blo = (int32_t)ceilf(fmaxf(blo - m, -fh));
-    w.bhi = (int32_t)floorf(fminf(bhi + m, fh));
-    return w;
-}
-
 // Calls f(entry, ray, kmin, hit, inv) for every entry of a unit's list and every ray
 // of the entry's window (window(entry)), a pair per thread: windows hold from
 // one ray to several hundred (near the camera), and with an entry per thread
-// or per warp a CTA would end with its widest.  In rounds of 256 entries,
-// whose windows are laid end to end.  CTA-cooperative.
+// or per warp a CTA would end with its widest.  In rounds of 256 entries (16
+// of the widest bundles), whose windows are laid end to end.  CTA-cooperative.
 struct PairSmem {
     uint32_t end[kThreads], first[kThreads], kmin[kThreads];
     uint16_t na[kThreads], entry[kThreads];
@@ -248,10 +153,10 @@ template <class L, class W, class F>
 __device__ __forceinline__ void for_pairs(const FrameArgs &a, const uint16_t *list, uint32_t n, PairSmem &ps,
                                           W window, F f) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t width = 2u * (uint32_t)a.hw + 1u;
-    for (uint32_t l0 = 0; l0 < n; l0 += kThreads) {
+    const uint32_t width = 2u * (uint32_t)a.hw + 1u, round = round_entries(a.ga.rays);
+    for (uint32_t l0 = 0; l0 < n; l0 += round) {
         uint32_t count = 0;
-        if (l0 + tid < n) {
+        if ((uint32_t)tid < round && l0 + tid < n) {
             const uint32_t e = list[l0 + tid];
             const Window w = window(e);
             count = (uint32_t)w.count();
@@ -290,7 +195,7 @@ __device__ __forceinline__ void for_pairs(const FrameArgs &a, const uint16_t *li
                 for (int d = kThreads / 2; d > 0; d >>= 1)
                     if (ps.end[at + d - 1] <= t) at += d;
                 const uint32_t q = t - (at ? ps.end[at - 1] : 0u), na = ps.na[at];
-                const uint32_t row = __float2uint_rz(__fdividef((float)q + 0.5f, (float)na));
+                const uint32_t row = row_of(q, na);
                 v[k] = at;
                 ray[k] = ps.first[at] + row * width + (q - row * na);
                 hit[k] = L::ld(a.ga.hit + ray[k]);

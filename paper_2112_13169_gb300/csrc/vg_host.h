@@ -259,7 +259,7 @@ inline void gather_setup(FrameArgs &a, uint8_t *base, size_t bytes) {
 
     const int64_t rays = (2 * (int64_t)a.hw + 1) * (2 * (int64_t)a.hh + 1);
     const int64_t tiles = (int64_t)((2 * a.hw + 8) >> 3) * ((2 * a.hh + 8) >> 3);
-    if (!base || rays * 20 + tiles * 4 + 2 * kNearWords * 4 > (int64_t)bytes || rays >= (int64_t(1) << 30)) return;
+    if (!base || rays * 20 + tiles * 4 + 2 * kNearWords * 4 > (int64_t)bytes || rays >= kMaxRays) return;
     g.rays = (int32_t)rays;
     g.inv = reinterpret_cast<float4 *>(base);
     g.hit = reinterpret_cast<uint32_t *>(g.inv + rays);

@@ -105,6 +105,7 @@ struct WordBox {
 constexpr int kNearReach = 7;            // voxels around the camera's that the rays mark themselves
 constexpr int kLateReach = 3;            // rays around each one whose latest hit is tabled
 constexpr int kNearWords = (2 * kNearReach + 1) * (2 * kNearReach + 1);
+constexpr int32_t kMaxRays = 1 << 27;    // of a gathered bundle (fewer)
 struct Gather {
     int32_t on;         // 0: the frame takes the scattered form (vg_rt.cuh)
     int32_t rays;       // rays of the bundle
