@@ -195,7 +195,7 @@ __device__ __forceinline__ void for_pairs(const FrameArgs &a, const uint16_t *li
                 for (int d = kThreads / 2; d > 0; d >>= 1)
                     if (ps.end[at + d - 1] <= t) at += d;
                 const uint32_t q = t - (at ? ps.end[at - 1] : 0u), na = ps.na[at];
-                const uint32_t row = row_of(q, na);
+                const uint32_t row = row_of(q, na, a.ga.rays);
                 v[k] = at;
                 ray[k] = ps.first[at] + row * width + (q - row * na);
                 hit[k] = L::ld(a.ga.hit + ray[k]);

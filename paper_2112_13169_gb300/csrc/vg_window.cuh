@@ -147,10 +147,10 @@ VG_BOTH uint32_t round_entries(int32_t rays) { return rays < (1 << 23) ? (uint32
 
 // q / na, the row of ray q of a window na rays wide.  (q + 1/2) / na lies at
 // least 1 / (2 na) from a whole number and the quotient within 2^-22 of
-// itself from it, so its whole part is exact below 2^21.  Windows past the
-// 2^20th ray, which only bundles of millions have, divide whole numbers.
-VG_BOTH uint32_t row_of(uint32_t q, uint32_t na) {
-    if (q >> 20) return q / na;
+// itself from it, so its whole part is exact below 2^21.  Bundles of 2^20 rays
+// and more divide whole numbers.
+VG_BOTH uint32_t row_of(uint32_t q, uint32_t na, int32_t rays) {
+    if (rays >> 20) return q / na;
     return (uint32_t)quotient((float)q + 0.5f, (float)na);
 }
 

@@ -51,13 +51,14 @@ def test_the_row_of_a_pair_is_exact(win):
     n2 = np.tile(na, 60)
     q, n2 = np.concatenate([q, q - 1, q + n2 // 2]).astype(np.uint32), np.tile(n2, 3)
     out = np.empty_like(q)
-    win.w_rows(C.c_int64(len(q)), ptr(q), ptr(n2), ptr(out))
-    assert np.array_equal(out, q // n2)
+    for rays in (1 << 20, 113_000_000, (1 << 20) - 1):
+        if rays < 1 << 20:                       # a window holds no more rays than the bundle
+            q, n2, out = (v[q < rays].copy() for v in (q, n2, out))
+        win.w_rows(C.c_int64(len(q)), ptr(q), ptr(n2), rays, ptr(out))
+        assert np.array_equal(out, q // n2)
     # the device's quotient is within two units in the last place: where it is
     # used, the row stays the same
-    small = q < 1 << 20
-    qs, ns = q[small], n2[small]
-    f = (qs.astype(np.float32) + np.float32(0.5)) / ns.astype(np.float32)
+    f = (q.astype(np.float32) + np.float32(0.5)) / n2.astype(np.float32)
     for to in (np.float32(0), np.float32(np.inf)):
         g = np.nextafter(np.nextafter(f, to), to)
-        assert np.array_equal(g.astype(np.uint32), qs // ns)
+        assert np.array_equal(g.astype(np.uint32), q // n2)

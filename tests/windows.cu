@@ -57,8 +57,8 @@ void w_voxels(int64_t m, const int32_t *i, int32_t *out) {
 
 uint32_t w_round_entries(int32_t rays) { return gather::round_entries(rays); }
 int32_t w_max_rays() { return kMaxRays; }
-void w_rows(int64_t m, const uint32_t *q, const uint32_t *na, uint32_t *out) {
-    for (int64_t j = 0; j < m; ++j) out[j] = gather::row_of(q[j], na[j]);
+void w_rows(int64_t m, const uint32_t *q, const uint32_t *na, int32_t rays, uint32_t *out) {
+    for (int64_t j = 0; j < m; ++j) out[j] = gather::row_of(q[j], na[j], rays);
 }
 
 }  // extern "C"
