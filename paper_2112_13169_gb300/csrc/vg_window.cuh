@@ -99,7 +99,9 @@ VG_BOTH Window window_of(const FrameArgs &a, const Place &p, float hx, float z) 
 }
 
 // The window of the face of voxel i that a walk enters through along axis k:
-// the projections of its corners, the margin beyond its edges.
+// the projections of its corners, the margin beyond its edges.  A word that
+// touches the bundle may hold voxels beside and behind the camera, where
+// corners have no projection: empty if the voxel lies outside the bundle.
 VG_BOTH Window face_window(const FrameArgs &a, const float S[3], const int32_t v0[3], const int32_t i[3], int k) {
     const Gather &g = a.ga;
     const float fvd = (float)a.vd, fw = (float)a.hw, fh = (float)a.hh;
@@ -116,6 +118,9 @@ VG_BOTH Window face_window(const FrameArgs &a, const float S[3], const int32_t v
     const float zn = p.c2 + fminf(u2, 0.0f) + fminf(w2, 0.0f) - g.m;
     w.kmin = bits_of(fminf(fmaxf(quotient(zn, fvd), 0.0f), 1.0f)) << 2;
     if (zn < 0.2f) {
+        if (!in_bundle(a, place_of(g, (float)i[0] + 0.5f - S[0], (float)i[1] + 0.5f - S[1], (float)i[2] + 0.5f - S[2]), g.ev,
+                       g.zv))
+            return Window{0, -1, 0, -1, 0};
         w.alo = -a.hw; w.ahi = a.hw; w.blo = -a.hh; w.bhi = a.hh;
         return w;
     }
