@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
                     gather::gather_unit<kGatherWords, false, units::LoadPlain>(
                         s_a, S, v0, (uint32_t)local, box, *reinterpret_cast<gather::GatherSmem<kGatherWords> *>(dyn));
                 } else {
-                    gather::slab_word(s_a, (local - box) * kThreads + threadIdx.x);
+                    gather::outside_word<false>(s_a, (local - box) * kThreads + threadIdx.x);
                 }
                 continue;
             }

@@ -30,8 +30,8 @@ __global__ void __launch_bounds__(kThreads) k_raylate(const FrameArgs a) {
     late_unit<units::LoadRO>(a, blockIdx.x, sh);
 }
 
-// The first `nbox` CTAs take the words of the frame's box, the others what a
-// re-centre brought in outside it.
+// The first `nbox` CTAs take the words of the frame's box, the others what
+// lies outside it: what a re-centre brought in, and a cloud's points.
 template <int WPU>
 __global__ void __launch_bounds__(kThreads) k_gather(const FrameArgs a, const int nbox) {
     __shared__ GatherSmem<WPU> sh;
@@ -41,13 +41,14 @@ __global__ void __launch_bounds__(kThreads) k_gather(const FrameArgs a, const in
     frame_start(a, S, v0);
     pdl_wait();
     if ((int)blockIdx.x < nbox) gather_unit<WPU, true, units::LoadPlain>(a, S, v0, blockIdx.x, nbox, sh);
-    else slab_word(a, (int64_t)((int)blockIdx.x - nbox) * kThreads + threadIdx.x);
+    else if (a.whole) outside_word<true>(a, (int64_t)((int)blockIdx.x - nbox) * kThreads + threadIdx.x);
+    else outside_word<false>(a, (int64_t)((int)blockIdx.x - nbox) * kThreads + threadIdx.x);
 }
 
 template <int WPU>
 cudaError_t gather_words(const FrameArgs &a, cudaStream_t s) {
     const unsigned nbox = word_units<WPU, 4>(a.box);
-    return launch_pdl(k_gather<WPU>, nbox + (unsigned)slab_units(a, kThreads), kThreads, 0, s, a, (int)nbox);
+    return launch_pdl(k_gather<WPU>, nbox + (unsigned)outside_units(a, kThreads), kThreads, 0, s, a, (int)nbox);
 }
 
 }  // namespace

@@ -92,9 +92,11 @@ __global__ void __launch_bounds__(256) k_inflate_tma(const __grid_constant__ CUt
     units::inflate_passes<R, TXW, TY, TZ>(g, out, r, tx, ty, tz, sm, BW, 3, sm + tma_box_words<TXW, TY, TZ>(r));
 }
 
-// The tiles of the frame's box: the first one and how many each way.
+// The tiles of what the frame can occupy, its box or (a cloud) the grid: the
+// first one and how many each way.
 template <int TXW, int TY, int TZ>
-dim3 box_tiles(const WordBox &b, int3 &t0) {
+dim3 box_tiles(const FrameArgs &a, int3 &t0) {
+    const WordBox b = a.whole ? WordBox{0, a.g.wx, 0, a.g.ny, 0, a.g.nz} : a.box;
     t0 = make_int3(b.w0 / TXW, b.y0 / TY, b.z0 / TZ);
     return dim3((b.w0 + b.nw + TXW - 1) / TXW - t0.x, (b.y0 + b.ny + TY - 1) / TY - t0.y,
                 (b.z0 + b.nz + TZ - 1) / TZ - t0.z);
@@ -103,7 +105,7 @@ dim3 box_tiles(const WordBox &b, int3 &t0) {
 template <int R, int TXW, int TY, int TZ>
 cudaError_t run(const FrameArgs &a, cudaStream_t s) {
     int3 t0;
-    const dim3 grid = box_tiles<TXW, TY, TZ>(a.box, t0);
+    const dim3 grid = box_tiles<TXW, TY, TZ>(a, t0);
     const size_t bytes = sizeof(uint32_t) * units::inflate_smem_words<R, TXW, TY, TZ>(a.r);
     return launch_pdl(k_inflate<R, TXW, TY, TZ>, grid, 256, bytes, s, a.g, (const uint32_t *)a.pl.occ_raw,
                       a.pl.occ_inf, a.r, t0);
@@ -181,7 +183,7 @@ cudaError_t run_tma(const FrameArgs &a, cudaStream_t s) {
     CUtensorMap m;
     if (!plane_map(a.pl.occ_raw, a.g, TXW + 8, TY + 2 * a.r, TZ + 2 * a.r, m)) return run<R, TXW, TY, TZ>(a, s);
     int3 t0;
-    const dim3 grid = box_tiles<TXW, TY, TZ>(a.box, t0);
+    const dim3 grid = box_tiles<TXW, TY, TZ>(a, t0);
     const size_t bytes = sizeof(uint32_t) * (tma_box_words<TXW, TY, TZ>(a.r) + (TZ + 2 * a.r) * (TY + 2 * a.r) * TXW);
     return launch_pdl(k_inflate_tma<R, TXW, TY, TZ>, grid, 256, bytes, s, m, a.g, a.pl.occ_inf, a.r, t0);
 }
@@ -241,7 +243,7 @@ cudaError_t launch_inflate(const FrameArgs &a, cudaStream_t s, const Sched &sc) 
     int tile = sc.inflate_tile;
     if (tile == kTileAuto) {
         int3 t0;
-        const dim3 t = wide_ok ? box_tiles<8, 8, 8>(a.box, t0) : box_tiles<4, 8, 8>(a.box, t0);
+        const dim3 t = wide_ok ? box_tiles<8, 8, 8>(a, t0) : box_tiles<4, 8, 8>(a, t0);
         const int64_t tiles8 = (int64_t)t.x * t.y * t.z;
         const int64_t sms = sms_of_current_device();
         const bool short_tiles = tiles8 >= sms && tiles8 < 4 * sms;

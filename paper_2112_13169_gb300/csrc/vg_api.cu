@@ -664,6 +664,7 @@ int vg_integrate_points(vg_grid *G, const float *xyz, int32_t mem, int64_t n, co
     FrameArgs a = frame_args(G, T);
     a.xyz = static_cast<const float *>(dptr);
     a.npts = n;
+    vg::host::cloud_box(a);
     gather_form(G, a);
     cudaError_t e = launch(G, VG_K_VOXELIZE, s, [&] { return vg::launch_voxelize_points(a, s, G->sched); });
     if (e == cudaSuccess) e = finish_frame(G, a, s);
@@ -964,7 +965,7 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
             it.skin_units = (int32_t)vg::gather::word_units<256, 1>(box);
             it.box_units = (int32_t)vg::gather::word_units<vg::kBatchGatherWords, 4>(box);
             units[0] += (vg::gather::table_threads(it.a) + 255) / 256;
-            units[3] = it.box_units + vg::gather::slab_units(it.a, 256);
+            units[3] = it.box_units + vg::gather::outside_units(it.a, 256);
             units[4] = it.near_units + it.skin_units;
             units[5] = vg::gather::late_units(it.a);
         } else {

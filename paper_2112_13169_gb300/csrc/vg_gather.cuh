@@ -801,31 +801,43 @@ __device__ __forceinline__ void gather_unit(const FrameArgs &a, const float S[3]
     __syncthreads();   // the shared memory may be reused right away
 }
 
-// The voxels a re-centre brought in outside the frame's box: words of the
-// slabs it brought in along x, y and z, a word per thread; the box's own are
-// gather_unit's.  Words in two slabs are written twice, alike.
-__host__ __device__ inline int64_t slab_words(const FrameArgs &a, int64_t part[3]) {
+// What lies outside the frame's box, a word per thread; the box's own words
+// are gather_unit's.  The voxels a re-centre brought in: words of the slabs it
+// brought in along x, y and z (words in two slabs are written twice, alike).
+// A cloud's points too (`whole`): all words of the grid.  Its box holds the
+// rays alone, since gathering a word costs more than merging it: 300,000 points
+// around the robot into 400 x 400 x 120 voxels took 65 us a frame with the grid
+// as the box.
+__host__ __device__ inline int64_t outside_words(const FrameArgs &a, int64_t part[3]) {
     const Ring &R = a.ring;
     const int64_t used = (a.g.nx + 31) / 32;
+    const WordBox &b = a.box;
+    part[0] = part[1] = part[2] = 0;
+    if (b.w0 == 0 && b.nw >= used && b.ny == a.g.ny && b.nz == a.g.nz) return 0;
+    if (a.whole) return used * a.g.ny * a.g.nz;
     part[0] = R.ehi[0] > R.elo[0] ? (int64_t)((R.ehi[0] + 31) / 32 - R.elo[0] / 32) * a.g.ny * a.g.nz : 0;
     part[1] = (int64_t)(R.ehi[1] - R.elo[1]) * used * a.g.nz;
     part[2] = (int64_t)(R.ehi[2] - R.elo[2]) * used * a.g.ny;
-    const WordBox &b = a.box;
-    if (b.w0 == 0 && b.nw >= used && b.ny == a.g.ny && b.nz == a.g.nz) part[0] = part[1] = part[2] = 0;
     return part[0] + part[1] + part[2];
 }
-__host__ __device__ inline int64_t slab_units(const FrameArgs &a, int threads) {
+__host__ __device__ inline int64_t outside_units(const FrameArgs &a, int threads) {
     int64_t part[3];
-    return (slab_words(a, part) + threads - 1) / threads;
+    return (outside_words(a, part) + threads - 1) / threads;
 }
 
-__device__ __forceinline__ void slab_word(const FrameArgs &a, int64_t t) {
+template <bool WHOLE>
+__device__ __forceinline__ void outside_word(const FrameArgs &a, int64_t t) {
     const Ring &R = a.ring;
     int64_t part[3];
-    if (t >= slab_words(a, part)) return;
+    if (t >= outside_words(a, part)) return;
     const uint32_t used = (uint32_t)(a.g.nx + 31) / 32u;
     int32_t i[3];
-    if (t < part[0]) {
+    if (WHOLE) {
+        const uint32_t row = (uint32_t)t / used;   // grids hold fewer than 2^27 words
+        i[0] = (int32_t)((uint32_t)t - row * used) * 32;
+        i[2] = (int32_t)(row / (uint32_t)a.g.ny);
+        i[1] = (int32_t)(row - (uint32_t)i[2] * (uint32_t)a.g.ny);
+    } else if (t < part[0]) {
         const uint32_t nw = (uint32_t)((R.ehi[0] + 31) / 32 - R.elo[0] / 32), row = (uint32_t)t / nw;
         i[0] = (R.elo[0] / 32 + (int32_t)((uint32_t)t - row * nw)) * 32;
         i[2] = (int32_t)(row / (uint32_t)a.g.ny);
@@ -844,16 +856,24 @@ __device__ __forceinline__ void slab_word(const FrameArgs &a, int64_t t) {
     if ((uint32_t)((i[0] >> 5) - b.w0) < (uint32_t)b.nw && (uint32_t)(i[1] - b.y0) < (uint32_t)b.ny &&
         (uint32_t)(i[2] - b.z0) < (uint32_t)b.nz)
         return;
+    const uint32_t w = word_of(a.g, i);
+    const uint32_t oc = WHOLE ? a.pl.occ_inf[w] : 0u;
     const int nbits = min(32, a.g.nx - i[0]);
-    const uint32_t ent = units::entering_bits(R, i[0], i[1], i[2], nbits);
-    if (ent == 0) return;
-    constexpr uint32_t kUnknown[9] = {};
+    const uint32_t touch = oc | units::entering_bits(R, i[0], i[1], i[2], nbits);
+    if (touch == 0) return;
+    uint32_t codes[9] = {};   // unknown
+    if (WHOLE && oc) {
+#pragma unroll
+        for (int m = 0; m < 8; ++m) codes[m] = units::merge4(oc, 0u, oc, m, 0u);
+        a.pl.occ_inf[w] = 0;
+        a.pl.occ_raw[w] = 0;
+    }
     uint8_t *rowp = a.loc + ((int64_t)units::ring_at(i[2], R.r[2], a.g.nz) * a.g.ny +
                              units::ring_at(i[1], R.r[1], a.g.ny)) * a.g.nx;
     const int32_t xb = units::ring_at(i[0], R.r[0], a.g.nx);
     const int n1 = min(nbits, a.g.nx - xb);
-    units::store_codes(rowp + xb, 0, n1, kUnknown, ent);
-    if (n1 < nbits) units::store_codes(rowp, n1, nbits, kUnknown, ent);
+    units::store_codes(rowp + xb, 0, n1, codes, touch);
+    if (n1 < nbits) units::store_codes(rowp, n1, nbits, codes, touch);
 }
 
 }  // namespace gather

@@ -168,23 +168,20 @@ inline void set_depth_frame(FrameArgs &a, const vg_params *p, const void *depth,
     depth_box(a, p, tx, ty);
 }
 
-// Narrows a depth frame's box to what its pixels (inflated by vox_inf) and
-// rays can reach: the pyramid of both from the camera, with two voxels to
-// spare for rounding (tx, ty: the tangents of half its fields of view).  Poses whose rotation block is no rotation keep their
-// linear map, so the corners bound it all the same.
-inline void depth_box(FrameArgs &a, const vg_params *p, double tx, double ty) {
-    const double d = std::max((double)a.vd, (double)p->depth / (double)p->vox_size);
-    const double kx = std::max(tx, a.vd > 0 ? (double)a.hw / a.vd : 0.0) * d;
-    const double ky = std::max(ty, a.vd > 0 ? (double)a.hh / a.vd : 0.0) * d;
+// Narrows a frame's box to a pyramid from the camera, of depth d voxels and
+// half sides kx and ky there, with `spare` voxels more for rounding.  Poses
+// whose rotation block is no rotation keep their linear map, so the corners
+// bound it all the same.
+inline void pyramid_box(FrameArgs &a, double d, double kx, double ky, double spare) {
     int32_t lo[3], hi[3];
     const int32_t n[3] = {a.g.nx, a.g.ny, a.g.nz};
     for (int k = 0; k < 3; ++k) {
         const double s = (double)a.T.t[k] / (double)a.vs;
         const double fwd = (double)a.T.R[k * 3 + 2] * d;
         const double side = std::fabs((double)a.T.R[k * 3]) * kx + std::fabs((double)a.T.R[k * 3 + 1]) * ky;
-        const double spare = a.r + 2.0 + 1e-6 * (std::fabs(s) + std::fabs(fwd) + side);
-        lo[k] = (int32_t)std::min(std::max(floor(s + std::min(0.0, fwd - side) - spare), 0.0), (double)n[k]);
-        hi[k] = (int32_t)std::min(std::max(ceil(s + std::max(0.0, fwd + side) + spare), 0.0), (double)n[k]);
+        const double m = spare + 1e-6 * (std::fabs(s) + std::fabs(fwd) + side);
+        lo[k] = (int32_t)std::min(std::max(floor(s + std::min(0.0, fwd - side) - m), 0.0), (double)n[k]);
+        hi[k] = (int32_t)std::min(std::max(ceil(s + std::max(0.0, fwd + side) + m), 0.0), (double)n[k]);
         if (hi[k] < lo[k]) hi[k] = lo[k];
     }
     if (lo[0] == hi[0] || lo[1] == hi[1] || lo[2] == hi[2]) {   // nothing of the grid: one word, for the launches
@@ -192,6 +189,21 @@ inline void depth_box(FrameArgs &a, const vg_params *p, double tx, double ty) {
         return;
     }
     a.box = {lo[0] / 32, (hi[0] + 31) / 32 - lo[0] / 32, lo[1], hi[1] - lo[1], lo[2], hi[2] - lo[2]};
+}
+
+// A depth frame's box: what its pixels (inflated by vox_inf) and rays can
+// reach (tx, ty: the tangents of half its fields of view).
+inline void depth_box(FrameArgs &a, const vg_params *p, double tx, double ty) {
+    const double d = std::max((double)a.vd, (double)p->depth / (double)p->vox_size);
+    const double kx = std::max(tx, a.vd > 0 ? (double)a.hw / a.vd : 0.0) * d;
+    const double ky = std::max(ty, a.vd > 0 ? (double)a.hh / a.vd : 0.0) * d;
+    pyramid_box(a, d, kx, ky, a.r + 2.0);
+}
+
+// A cloud's box: what its rays can reach.  Its points lie anywhere.
+inline void cloud_box(FrameArgs &a) {
+    a.whole = 1;
+    pyramid_box(a, a.vd, a.hw, a.hh, 2.0);
 }
 
 // Whether the gathered form of a frame (vg_gather.cuh) is the faster one:

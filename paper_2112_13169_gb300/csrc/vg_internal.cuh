@@ -93,7 +93,8 @@ struct Ring {
 };
 
 // The part of a grid a frame can mark or occupy: words [w0, w0 + nw) of rows
-// [y0, y0 + ny) of slices [z0, z0 + nz).  Everything outside is unoccupied.
+// [y0, y0 + ny) of slices [z0, z0 + nz).  Everything outside is unoccupied,
+// but for a cloud's points (FrameArgs::whole).
 struct WordBox {
     int32_t w0, nw, y0, ny, z0, nz;
 };
@@ -144,6 +145,7 @@ struct FrameArgs {
     Planes pl;
     uint8_t *loc;
     WordBox box;                // K2's tiles and the gathered form's words
+    int32_t whole;              // 1: the box bounds the rays alone, points may lie anywhere in the grid
     Ring ring;                  // loc's ring addressing, with the voxels a re-centre brought in
     unsigned long long *stats;  // NULL unless VG_FLAG_STATS
     uint32_t *rt_next;          // K3's counter of handed-out bundles, zeroed by K1; NULL: static only

@@ -151,3 +151,30 @@ def test_reads_through_the_ring(vg, n):
             o.loc[:] = src
             g.write(src, g.origin)
     g.close()
+
+
+# points all round the robot: outside the rays' box, where the merge takes
+# them, in words the box shares with the rays, and in what re-centres bring in
+@pytest.mark.parametrize("n,r,off", [((200, 200, 100), 2, 0.0), ((211, 173, 61), 0, 0.0), ((400, 130, 70), 5, 0.0),
+                                     ((200, 200, 100), 1, 4.9), ((200, 200, 100), 0, 60.0)])
+def test_gathered_clouds_all_round(vg, n, r, off):
+    rng = np.random.default_rng(sum(n) + r)
+    P = Grids(vg, n, 0.05, 87.0, 58.0, 5.0, r, (0.0, 0.0, 0.0))
+    half = np.array(n) * 0.05 / 2
+    for k in range(4):
+        # walls of a corridor, scattered points, and a few far outside the grid
+        w = rng.uniform(-1, 1, (20_000, 3)) * half
+        w[:8_000, 1] = np.sign(w[:8_000, 1])
+        w[8_000:14_000, 2] = -0.42
+        w[-500:] *= 3
+        T = body_pose([off + 0.01, -0.02, 0.03], [0.0, 0.0, 2.2, -1.4][k] + (np.pi if 0 < off < 5 else 0.0), 0.1 * k, 0.05 * k)
+        xyz = ((w - T[:3, 3]) @ T[:3, :3]).astype(np.float32)
+        P.g.integrate_points(torch.from_numpy(xyz).cuda(), T)
+        P.o.integrate_points(T, xyz)
+        if k != 1:                                        # (frame 2 merges a pending re-centre)
+            P.check("%s cloud %d" % (n, k))
+        to = np.array([0.4, -0.3, 0.2]) * (k + 1)
+        P.g.shift(to)
+        P.o.shift(to)
+    P.check("%s after the last re-centre" % (n,))
+    P.g.close()
