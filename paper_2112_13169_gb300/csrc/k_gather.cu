@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(kThreads) k_raylate(const FrameArgs a) {
     __shared__ LateSmem sh;
     pdl_trigger();
     pdl_wait();
-    late_unit<units::LoadRO>(a, blockIdx.x, sh);
+    late_unit<units::LoadPlain>(a, blockIdx.x, sh);
 }
 
 // The first `nbox` CTAs take the words of the frame's box, the others what

@@ -14,13 +14,13 @@ namespace vg {
 namespace {
 
 template <int R, int TXW, int TY, int TZ>
-__global__ void __launch_bounds__(256) k_inflate(const PlaneGeom g, const uint32_t *__restrict__ raw,
-                                                 uint32_t *__restrict__ out, const int r_rt, const int3 first) {
+__global__ void __launch_bounds__(256) k_inflate(const PlaneGeom g, const uint32_t *raw, uint32_t *out,
+                                                 const int r_rt, const int3 first) {
     extern __shared__ uint32_t sm[];
     pdl_trigger();
     pdl_wait();
-    units::inflate_tile<R, TXW, TY, TZ, units::LoadRO>(g, raw, out, r_rt, first.x + blockIdx.x, first.y + blockIdx.y,
-                                                       first.z + blockIdx.z, sm);
+    units::inflate_tile<R, TXW, TY, TZ, units::LoadPlain>(g, raw, out, r_rt, first.x + blockIdx.x, first.y + blockIdx.y,
+                                                          first.z + blockIdx.z, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -54,7 +54,7 @@ __host__ __device__ constexpr int tma_box_words(int r) { return (TXW + 8) * (TY 
 
 template <int R, int TXW, int TY, int TZ>
 __global__ void __launch_bounds__(256) k_inflate_tma(const __grid_constant__ CUtensorMap tm, const PlaneGeom g,
-                                                     uint32_t *__restrict__ out, const int r_rt, const int3 first) {
+                                                     uint32_t *out, const int r_rt, const int3 first) {
     constexpr int BW = TXW + 8;
     const int r = R > 0 ? R : r_rt;
     const uint32_t bytes = (uint32_t)tma_box_words<TXW, TY, TZ>(r) * 4u;

@@ -8,8 +8,7 @@ namespace vg {
 namespace {
 
 template <bool RL, int WPU>
-__global__ void __launch_bounds__(256) k_merge(const PlaneGeom g, Planes pl, uint8_t *__restrict__ loc,
-                                               const Ring ring) {
+__global__ void __launch_bounds__(256) k_merge(const PlaneGeom g, Planes pl, uint8_t *loc, const Ring ring) {
     pdl_trigger();
     pdl_wait();
 #pragma unroll
@@ -20,8 +19,8 @@ __global__ void __launch_bounds__(256) k_merge(const PlaneGeom g, Planes pl, uin
 // The literal loc_grid reading of Alg. 2: the occupied voxels of loc_grid
 // in the grid's own frame (voxels a re-centre brought in are unknown), as a
 // bit plane (one thread per plane word, every word written).
-__global__ void __launch_bounds__(256) k_loc_occupancy(const PlaneGeom g, const uint8_t *__restrict__ loc,
-                                                       const Ring R, uint32_t *__restrict__ out) {
+__global__ void __launch_bounds__(256) k_loc_occupancy(const PlaneGeom g, const uint8_t *loc, const Ring R,
+                                                       uint32_t *out) {
     pdl_trigger();
     pdl_wait();
     const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -36,17 +35,16 @@ __global__ void __launch_bounds__(256) k_loc_occupancy(const PlaneGeom g, const 
         const uint8_t *rowp =
             loc + ((int64_t)units::ring_at(z, R.r[2], g.nz) * g.ny + units::ring_at(y, R.r[1], g.ny)) * g.nx;
         for (int k = 0; k < nbits; ++k)
-            if (!((ent >> k) & 1u) && __ldg(rowp + units::ring_at(x0 + k, R.r[0], g.nx)) == 2)   // VG_OCC
+            if (!((ent >> k) & 1u) && rowp[units::ring_at(x0 + k, R.r[0], g.nx)] == 2)   // VG_OCC
                 bits |= 1u << k;
     }
     out[w] = bits;
 }
 
-__global__ void __launch_bounds__(256) k_shift(const PlaneGeom g, const Ring ring, const uint8_t *__restrict__ src,
-                                               uint8_t *__restrict__ dst) {
+__global__ void __launch_bounds__(256) k_shift(const PlaneGeom g, const Ring ring, const uint8_t *src, uint8_t *dst) {
     pdl_trigger();
     pdl_wait();
-    units::shift_chunk<units::LoadRO>(g, ring, src, dst, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    units::shift_chunk<units::LoadPlain>(g, ring, src, dst, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 template <int WPU>

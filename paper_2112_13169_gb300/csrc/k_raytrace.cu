@@ -26,8 +26,8 @@ __global__ void __launch_bounds__(kThreads, 5) k_raytrace(const FrameArgs a, con
     box_clear(box_fr, box_tr);
     const Pass1 p1 = rt_record(a, ln, b, buffered, buf);
     pdl_wait();
-    box_stage<units::LoadRO, false>(a, b, box_fr, box_tr, occ_box);
-    unsigned visits = rt_resolve<LPR, units::LoadRO, EXACT>(a, ln, b, p1, box_fr, box_tr, occ_box, buf);
+    box_stage<units::LoadPlain, false>(a, b, box_fr, box_tr, occ_box);
+    unsigned visits = rt_resolve<LPR, units::LoadPlain, EXACT>(a, ln, b, p1, box_fr, box_tr, occ_box, buf);
     if (a.rt_next && groups > (int64_t)gridDim.x) {
         // the groups past the launch's CTAs go out one bundle at a time, from
         // a counter in device memory (zeroed by this frame's K1), so that the
@@ -39,12 +39,12 @@ __global__ void __launch_bounds__(kThreads, 5) k_raytrace(const FrameArgs a, con
             t = __shfl_sync(kFull, t, 0);
             const int64_t grp = (int64_t)gridDim.x + t / kWarps;
             if (grp >= groups) break;
-            visits += rt_bundle<LPR, units::LoadRO, EXACT>(a, S, b, (int64_t)(t % kWarps) * groups + grp, buffered,
+            visits += rt_bundle<LPR, units::LoadPlain, EXACT>(a, S, b, (int64_t)(t % kWarps) * groups + grp, buffered,
                                                            box_fr, box_tr, occ_box, buf);
         }
     } else {
         for (int64_t grp = blockIdx.x + gridDim.x; grp < groups; grp += gridDim.x)
-            visits += rt_group<LPR, units::LoadRO, EXACT>(a, S, b, grp, groups, buffered, box_fr, box_tr, occ_box,
+            visits += rt_group<LPR, units::LoadPlain, EXACT>(a, S, b, grp, groups, buffered, box_fr, box_tr, occ_box,
                                                           buf);
     }
     box_flush(a, b, box_fr, box_tr);

@@ -2,12 +2,11 @@
 // unit of work, shared by the one-kernel-per-step launches (k_*.cu) and the
 // fused persistent launch (k_batch.cu).
 //
-// Loads of data that an earlier phase of the same launch may have written go
-// through a load policy: LoadRO (the read-only path, for one-step kernels
-// whose inputs were written by earlier launches and are not written by the
-// kernel), LoadPlain (ordinary loads, for data the kernel itself updates)
-// or LoadL2 (loads that skip the SM's L1, for phases of a fused launch that
-// read what other SMs wrote before a grid barrier).
+// Loads of data that an earlier launch or phase wrote go through a load
+// policy: LoadPlain (ordinary loads) or LoadL2 (loads that skip the SM's L1).
+// None take the read-only path: it is for data that nothing writes while the
+// kernel lives, and the one-step kernels are dependent launches, alive while
+// the kernel before them still writes.
 #pragma once
 
 #include "vg_internal.cuh"
@@ -16,11 +15,6 @@ namespace vg {
 namespace units {
 
 constexpr unsigned kFull = 0xffffffffu;
-
-struct LoadRO {
-    template <class T>
-    static __device__ __forceinline__ T ld(const T *p) { return __ldg(p); }
-};
 
 struct LoadPlain {
     template <class T>
@@ -212,10 +206,10 @@ __device__ __forceinline__ void load_depths(const FrameArgs &a, int32_t tile, in
     if (VEC) {
         if (u >= a.W) return;
         if (DT == 0) {
-            const float4 q = __ldg(reinterpret_cast<const float4 *>(a.depth) + (p0 >> 2));
+            const float4 q = reinterpret_cast<const float4 *>(a.depth)[p0 >> 2];
             d[0] = q.x; d[1] = q.y; d[2] = q.z; d[3] = q.w;
         } else {
-            const ushort4 q = __ldg(reinterpret_cast<const ushort4 *>(a.depth) + (p0 >> 2));
+            const ushort4 q = reinterpret_cast<const ushort4 *>(a.depth)[p0 >> 2];
             d[0] = __fmul_rn((float)q.x, a.scale);
             d[1] = __fmul_rn((float)q.y, a.scale);
             d[2] = __fmul_rn((float)q.z, a.scale);
@@ -225,8 +219,8 @@ __device__ __forceinline__ void load_depths(const FrameArgs &a, int32_t tile, in
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             if (u + j < a.W) {
-                if (DT == 0) d[j] = __ldg(reinterpret_cast<const float *>(a.depth) + p0 + j);
-                else d[j] = __fmul_rn((float)__ldg(reinterpret_cast<const uint16_t *>(a.depth) + p0 + j), a.scale);
+                if (DT == 0) d[j] = reinterpret_cast<const float *>(a.depth)[p0 + j];
+                else d[j] = __fmul_rn((float)reinterpret_cast<const uint16_t *>(a.depth)[p0 + j], a.scale);
             }
     }
 }
@@ -291,9 +285,9 @@ __device__ __forceinline__ void voxelize_run(const FrameArgs &a, int32_t tile, i
 // The word and bit of point i of the cloud (kNoWord past its end).
 __device__ __forceinline__ uint32_t point_of_cloud(const FrameArgs &a, int64_t i, uint32_t &bit) {
     if (i >= a.npts) return kNoWord;
-    const float x = __ldg(a.xyz + 3 * i + 0);
-    const float y = __ldg(a.xyz + 3 * i + 1);
-    const float z = __ldg(a.xyz + 3 * i + 2);
+    const float x = a.xyz[3 * i + 0];
+    const float y = a.xyz[3 * i + 1];
+    const float z = a.xyz[3 * i + 2];
     if (!(isfinite(x) && isfinite(y) && isfinite(z))) return kNoWord;
     return point_word(a, x, y, z, bit);
 }
