@@ -152,11 +152,15 @@ VG_BOTH uint32_t round_entries(int32_t rays) { return rays < (1 << 23) ? (uint32
 
 // q / na, the row of ray q of a window na rays wide.  (q + 1/2) / na lies at
 // least 1 / (2 na) from a whole number and the quotient within 2^-22 of
-// itself from it, so its whole part is exact below 2^21.  Bundles of 2^20 rays
-// and more divide whole numbers.
+// itself from it, so its whole part is exact below 2^21.  Windows of bundles
+// of 2^20 rays and more (fewer than 2^27, so off by one at most) are put right.
+VG_BOTH uint32_t put_right(uint32_t row, uint32_t q, uint32_t na) {
+    const int32_t left = (int32_t)(q - row * na);
+    return left < 0 ? row - 1u : row + (uint32_t)(left >= (int32_t)na);
+}
 VG_BOTH uint32_t row_of(uint32_t q, uint32_t na, int32_t rays) {
-    if (rays >> 20) return q / na;
-    return (uint32_t)quotient((float)q + 0.5f, (float)na);
+    const uint32_t row = (uint32_t)quotient((float)q + 0.5f, (float)na);
+    return rays >> 20 ? put_right(row, q, na) : row;
 }
 
 }  // namespace gather

@@ -56,12 +56,15 @@ def test_the_row_of_a_pair_is_exact(win):
             q, n2, out = (v[q < rays].copy() for v in (q, n2, out))
         win.w_rows(C.c_int64(len(q)), ptr(q), ptr(n2), rays, ptr(out))
         assert np.array_equal(out, q // n2)
-    # the device's quotient is within two units in the last place: where it is
-    # used, the row stays the same
-    f = (q.astype(np.float32) + np.float32(0.5)) / n2.astype(np.float32)
-    for to in (np.float32(0), np.float32(np.inf)):
-        g = np.nextafter(np.nextafter(f, to), to)
-        assert np.array_equal(g.astype(np.uint32), q // n2)
+        # the device's quotient is within two units in the last place: the row
+        # stays the same, or is put right
+        f = (q.astype(np.float32) + np.float32(0.5)) / n2.astype(np.float32)
+        for to in (np.float32(0), np.float32(np.inf)):
+            row = np.nextafter(np.nextafter(f, to), to).astype(np.uint32)
+            if rays >= 1 << 20:
+                assert (row != q // n2).any()
+                win.w_put_right(C.c_int64(len(q)), ptr(q), ptr(n2), ptr(row))
+            assert np.array_equal(row, q // n2)
 
 
 # ---------------------------------------------------------------------------

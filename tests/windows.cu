@@ -60,5 +60,8 @@ int32_t w_max_rays() { return kMaxRays; }
 void w_rows(int64_t m, const uint32_t *q, const uint32_t *na, int32_t rays, uint32_t *out) {
     for (int64_t j = 0; j < m; ++j) out[j] = gather::row_of(q[j], na[j], rays);
 }
+void w_put_right(int64_t m, const uint32_t *q, const uint32_t *na, uint32_t *row) {
+    for (int64_t j = 0; j < m; ++j) row[j] = gather::put_right(row[j], q[j], na[j]);
+}
 
 }  // extern "C"
