@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
             if (i != cur) {
                 __syncthreads();   // the previous frame's copy is no longer read
                 stage_args(items[i].a, s_a);
-                if (threadIdx.x == 0) s_kind = __ldg(&items[i].dtype) * 2 + __ldg(&items[i].vec);
+                if (threadIdx.x == 0) s_kind = __ldg(&items[i].dtype) * 3 + __ldg(&items[i].pix_mode);
                 __syncthreads();
                 cur = i;
             }
@@ -202,10 +202,12 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
             // the one before is placed
             const int run = (int)(hi - u < pix - local ? hi - u : pix - local);
             switch (s_kind) {
-            case 0: units::voxelize_run<0, false>(s_a, (int32_t)local, run, tab); break;
-            case 1: units::voxelize_run<0, true>(s_a, (int32_t)local, run, tab); break;
-            case 2: units::voxelize_run<1, false>(s_a, (int32_t)local, run, tab); break;
-            default: units::voxelize_run<1, true>(s_a, (int32_t)local, run, tab); break;
+            case 0: units::voxelize_run<0, units::kPixTile>(s_a, (int32_t)local, run, tab); break;
+            case 1: units::voxelize_run<0, units::kPixTile4>(s_a, (int32_t)local, run, tab); break;
+            case 2: units::voxelize_run<0, units::kPixLinear>(s_a, (int32_t)local, run, tab); break;
+            case 3: units::voxelize_run<1, units::kPixTile>(s_a, (int32_t)local, run, tab); break;
+            case 4: units::voxelize_run<1, units::kPixTile4>(s_a, (int32_t)local, run, tab); break;
+            default: units::voxelize_run<1, units::kPixLinear>(s_a, (int32_t)local, run, tab); break;
             }
             u += run;
         }

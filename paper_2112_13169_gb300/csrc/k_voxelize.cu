@@ -13,7 +13,7 @@ namespace {
 // slots to K3's CTAs, whose walk runs before they wait for K2.
 //
 // The first `ntab` CTAs write the gathered form's ray table instead.
-template <int DT, bool VEC>
+template <int DT, int MODE>
 __global__ void __launch_bounds__(256) k_voxelize_depth(const FrameArgs a, const int early, const int ntab) {
     __shared__ units::WordTab tab;
     pdl_wait();   // the depth image and the planes belong to earlier work
@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(256) k_voxelize_depth(const FrameArgs a, const
     }
     const unsigned block = blockIdx.x - ntab;
     if (a.rt_next && block == 0 && threadIdx.x == 0) *a.rt_next = 0u;   // K3 of this frame counts from 0
-    units::voxelize_tile<DT, VEC>(a, (int32_t)block, tab);
+    units::voxelize_tile<DT, MODE>(a, (int32_t)block, tab);
 }
 
 __global__ void __launch_bounds__(256) k_voxelize_points(const FrameArgs a, const int early, const int ntab) {
@@ -85,15 +85,17 @@ constexpr int64_t kDenseBlocks = 152;   // one to an SM
 }  // namespace
 
 cudaError_t launch_voxelize_depth(const FrameArgs &a, int32_t dtype, cudaStream_t s, const Sched &sc) {
-    const int early = sc.early_inflate;
     const int ntab = (int)((gather::table_threads(a) + 255) / 256);
-    const unsigned blocks = (unsigned)units::pixel_tiles(a.W, a.H) + ntab;
-    if (dtype == 0) {
-        if (units::pixels_aligned(a.depth, a.W, 4)) return launch_pdl(k_voxelize_depth<0, true>, blocks, 256, 0, s, a, early, ntab);
-        return launch_pdl(k_voxelize_depth<0, false>, blocks, 256, 0, s, a, early, ntab);
+    const unsigned blocks = (unsigned)units::pixel_tiles(a) + ntab;
+    auto run = [&](void (*k)(FrameArgs, int, int)) { return launch_pdl(k, blocks, 256, 0, s, a, (int)sc.early_inflate, ntab); };
+    switch (dtype * 3 + units::pixel_mode(a, dtype == 0 ? 4 : 2)) {
+    case 0: return run(k_voxelize_depth<0, units::kPixTile>);
+    case 1: return run(k_voxelize_depth<0, units::kPixTile4>);
+    case 2: return run(k_voxelize_depth<0, units::kPixLinear>);
+    case 3: return run(k_voxelize_depth<1, units::kPixTile>);
+    case 4: return run(k_voxelize_depth<1, units::kPixTile4>);
+    default: return run(k_voxelize_depth<1, units::kPixLinear>);
     }
-    if (units::pixels_aligned(a.depth, a.W, 2)) return launch_pdl(k_voxelize_depth<1, true>, blocks, 256, 0, s, a, early, ntab);
-    return launch_pdl(k_voxelize_depth<1, false>, blocks, 256, 0, s, a, early, ntab);
 }
 
 cudaError_t launch_voxelize_points(const FrameArgs &a, cudaStream_t s, const Sched &sc) {

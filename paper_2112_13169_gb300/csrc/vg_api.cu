@@ -944,7 +944,7 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
         if (G->p.vox_inf == 0) it.a.pl.occ_inf = it.a.pl.occ_raw;
         it.a.occ_test = it.a.pl.occ_inf;
         it.dtype = f.dtype;
-        it.vec = vg::units::pixels_aligned(f.depth, f.width, f.dtype == VG_DEPTH_F32 ? 4 : 2);
+        it.pix_mode = vg::units::pixel_mode(it.a, f.dtype == VG_DEPTH_F32 ? 4 : 2);
         int lpr = B->lanes ? B->lanes : (G->lanes_per_ray ? G->lanes_per_ray : vg::auto_lanes_per_ray(G->vd, G->hw, G->hh));
         it.lpr = lpr < 8 ? 8 : lpr;
         it.txw = G->g.wx % 8 == 0 ? 8 : 4;
@@ -958,7 +958,7 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
         }
         it.buffered = G->g.words < vg::kRunWords ? 1 : 0;
         const int64_t nrays = (2 * (int64_t)G->hw + 1) * (2 * (int64_t)G->hh + 1);
-        it.pix_units = vg::units::pixel_tiles(f.width, f.height);
+        it.pix_units = vg::units::pixel_tiles(it.a);
         int64_t units[6] = {it.pix_units, G->p.vox_inf > 0 ? (int64_t)it.tiles[0] * it.tiles[1] * it.tiles[2] : 0};
         if (it.a.ga.on) {
             it.near_units = vg::gather::near_units_of(it.a);

@@ -135,6 +135,7 @@ struct FrameArgs {
     int32_t W, H;
     float scale;       // u16 -> metres
     float fx, fy, cx, cy;
+    int32_t linear;    // 1: K1 takes the pixels as they lie in memory, not in tiles (vg_units.cuh)
     float rvs, rfx, rfy;        // reciprocals for K1's divisions (host::reciprocal)
     // point cloud input
     const float *xyz;
@@ -167,7 +168,7 @@ struct BatchItem {
     int32_t tile0[3];   // the first of them
     int32_t pix_units;  // phase 1: units of pixels; the others write the ray table
     int32_t dtype;      // 0 f32, 1 u16
-    int32_t vec;        // depth base aligned for 4-pixel loads
+    int32_t pix_mode;   // units::pixel_mode
     int32_t lpr;        // K3 lanes per ray: 8, 16 or 32
     int32_t txw;        // inflate tile width in words: 4 or 8
     int32_t tz;         // inflate tile height in slices: 4 or 8

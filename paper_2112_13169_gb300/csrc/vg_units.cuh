@@ -178,24 +178,68 @@ __device__ __forceinline__ void tab_flush(WordTab &tab, uint32_t *plane) {
     }
 }
 
-// The image in tiles of kTileW x kTileH pixels, four of a row to a thread.
-constexpr int kTileW = 32, kTileH = 32, kTileLanes = kTileW / 4;
+// The image in tiles of kTileW x kTileH pixels, four of a row to a thread, or
+// (FrameArgs::linear) of kTilePixels pixels as they lie in memory.
+constexpr int kTileW = 32, kTileH = 32, kTileLanes = kTileW / 4, kTilePixels = kTileW * kTileH;
 static_assert(kTileLanes * kTileH == 256, "a thread per four pixels");
 __host__ __device__ inline int32_t pixel_tiles_x(int32_t W) { return (W - 1) / kTileW + 1; }
-__host__ __device__ inline int32_t pixel_tiles(int32_t W, int32_t H) {
-    return pixel_tiles_x(W) * ((H - 1) / kTileH + 1);
+__host__ __device__ inline int32_t pixel_tiles(const FrameArgs &a) {
+    if (a.linear) return (int32_t)(((int64_t)a.W * a.H - 1) / kTilePixels + 1);
+    return pixel_tiles_x(a.W) * ((a.H - 1) / kTileH + 1);
 }
 
-// Whether every four pixels from a fourth column on can be loaded at once.
-__host__ __device__ inline bool pixels_aligned(const void *depth, int32_t W, int bytes) {
-    return W % 4 == 0 && reinterpret_cast<uintptr_t>(depth) % (4u * (unsigned)bytes) == 0;
+// Whether every whole four of the image's pixels can be loaded at once.
+__host__ __device__ inline bool pixels_aligned(const void *depth, int bytes) {
+    return reinterpret_cast<uintptr_t>(depth) % (4u * (unsigned)bytes) == 0;
+}
+
+// How K1 takes an image's pixels: in tiles one by one, in tiles by fours, or
+// (kPixLinear) as they lie, by fours where the image's address allows it.
+enum { kPixTile = 0, kPixTile4 = 1, kPixLinear = 2 };
+__host__ __device__ inline int pixel_mode(const FrameArgs &a, int bytes) {
+    if (a.linear) return kPixLinear;
+    return a.W % 4 == 0 && pixels_aligned(a.depth, bytes) ? kPixTile4 : kPixTile;
+}
+
+// Four pixels at once.
+template <int DT>
+__device__ __forceinline__ void load_four(const FrameArgs &a, uint32_t p0, float d[4]) {
+    if (DT == 0) {
+        const float4 q = reinterpret_cast<const float4 *>(a.depth)[p0 >> 2];
+        d[0] = q.x; d[1] = q.y; d[2] = q.z; d[3] = q.w;
+    } else {
+        const ushort4 q = reinterpret_cast<const ushort4 *>(a.depth)[p0 >> 2];
+        d[0] = __fmul_rn((float)q.x, a.scale);
+        d[1] = __fmul_rn((float)q.y, a.scale);
+        d[2] = __fmul_rn((float)q.z, a.scale);
+        d[3] = __fmul_rn((float)q.w, a.scale);
+    }
+}
+
+// One pixel.
+template <int DT>
+__device__ __forceinline__ float load_one(const FrameArgs &a, uint32_t p) {
+    if (DT == 0) return reinterpret_cast<const float *>(a.depth)[p];
+    return __fmul_rn((float)reinterpret_cast<const uint16_t *>(a.depth)[p], a.scale);
 }
 
 // The depths of the thread's pixels u .. u+3 of row v of a tile (0 outside
-// the image).  DT: 0 = f32, 1 = u16.  VEC: the image's base and rows are
-// aligned for a 4-pixel load.
-template <int DT, bool VEC>
+// the image), or of the four from (u, v) on of a linear one.  DT: 0 = f32, 1 =
+// u16.  MODE: pixel_mode.
+template <int DT, int MODE>
 __device__ __forceinline__ void load_depths(const FrameArgs &a, int32_t tile, int32_t &u, int32_t &v, float d[4]) {
+    if (MODE == kPixLinear) {
+        const uint32_t p = (uint32_t)tile * (uint32_t)kTilePixels + threadIdx.x * 4u, n = (uint32_t)a.W * (uint32_t)a.H;
+        v = (int32_t)(p / (uint32_t)a.W);
+        u = (int32_t)(p - (uint32_t)v * (uint32_t)a.W);
+        if (p + 4u <= n && pixels_aligned(a.depth, DT == 0 ? 4 : 2)) {
+            load_four<DT>(a, p, d);
+            return;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) d[j] = p + j < n ? load_one<DT>(a, p + j) : 0.0f;
+        return;
+    }
     const int32_t tx = pixel_tiles_x(a.W), ty = tile / tx;
     u = (tile - ty * tx) * kTileW + (int32_t)(threadIdx.x % kTileLanes) * 4;
     v = ty * kTileH + (int32_t)(threadIdx.x / kTileLanes);
@@ -203,38 +247,30 @@ __device__ __forceinline__ void load_depths(const FrameArgs &a, int32_t tile, in
 #pragma unroll
     for (int j = 0; j < 4; ++j) d[j] = 0.0f;
     if (v >= a.H) return;
-    if (VEC) {
-        if (u >= a.W) return;
-        if (DT == 0) {
-            const float4 q = reinterpret_cast<const float4 *>(a.depth)[p0 >> 2];
-            d[0] = q.x; d[1] = q.y; d[2] = q.z; d[3] = q.w;
-        } else {
-            const ushort4 q = reinterpret_cast<const ushort4 *>(a.depth)[p0 >> 2];
-            d[0] = __fmul_rn((float)q.x, a.scale);
-            d[1] = __fmul_rn((float)q.y, a.scale);
-            d[2] = __fmul_rn((float)q.z, a.scale);
-            d[3] = __fmul_rn((float)q.w, a.scale);
-        }
+    if (MODE == kPixTile4) {
+        if (u < a.W) load_four<DT>(a, p0, d);
     } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            if (u + j < a.W) {
-                if (DT == 0) d[j] = reinterpret_cast<const float *>(a.depth)[p0 + j];
-                else d[j] = __fmul_rn((float)reinterpret_cast<const uint16_t *>(a.depth)[p0 + j], a.scale);
-            }
+            if (u + j < a.W) d[j] = load_one<DT>(a, p0 + j);
     }
 }
 
 // Sets the thread's pixels, of depths d (outside the image: 0, which sets
-// nothing), in the table.  Warp-synchronous.
+// nothing), in the table.  LIN: they go on in the next row.  Warp-synchronous.
+template <bool LIN>
 __device__ __forceinline__ void voxelize_depths(const FrameArgs &a, int32_t u, int32_t v, const float d[4], WordTab &tab) {
     uint32_t key[4], bit[4];
     unsigned kept = 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         bit[j] = 0;
-        key[j] = pixel_word(a, d[j], u + j, v, bit[j]);
+        key[j] = pixel_word(a, d[j], LIN ? u : u + j, v, bit[j]);
         kept += (key[j] != kNoWord);
+        if (LIN && ++u == a.W) {
+            u = 0;
+            ++v;
+        }
     }
     // neighbouring pixels often share a word: once for a run of the thread's
 #pragma unroll
@@ -250,32 +286,32 @@ __device__ __forceinline__ void voxelize_depths(const FrameArgs &a, int32_t u, i
 }
 
 // One tile.  CTA-cooperative (256 threads).
-template <int DT, bool VEC>
+template <int DT, int MODE>
 __device__ __forceinline__ void voxelize_tile(const FrameArgs &a, int32_t tile, WordTab &tab) {
     float d[4];
     int32_t u, v;
-    load_depths<DT, VEC>(a, tile, u, v, d);
+    load_depths<DT, MODE>(a, tile, u, v, d);
     tab_clear(tab);
     __syncthreads();
-    voxelize_depths(a, u, v, d, tab);
+    voxelize_depths<MODE == kPixLinear>(a, u, v, d, tab);
     __syncthreads();
     tab_flush(tab, a.pl.occ_raw);
 }
 
 // `tiles` tiles from `tile` on, each one's depths loaded while the one before
 // is placed; finds the table clear and leaves it so.  CTA-cooperative.
-template <int DT, bool VEC>
+template <int DT, int MODE>
 __device__ __forceinline__ void voxelize_run(const FrameArgs &a, int32_t tile, int32_t tiles, WordTab &tab) {
     float d[4], next[4];
     int32_t u, v, un, vn;
-    load_depths<DT, VEC>(a, tile, un, vn, next);
+    load_depths<DT, MODE>(a, tile, un, vn, next);
     for (int32_t k = 0; k < tiles; ++k) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) d[j] = next[j];
         u = un;
         v = vn;
-        if (k + 1 < tiles) load_depths<DT, VEC>(a, tile + k + 1, un, vn, next);
-        voxelize_depths(a, u, v, d, tab);
+        if (k + 1 < tiles) load_depths<DT, MODE>(a, tile + k + 1, un, vn, next);
+        voxelize_depths<MODE == kPixLinear>(a, u, v, d, tab);
         __syncthreads();
         tab_flush(tab, a.pl.occ_raw);
         __syncthreads();
@@ -292,7 +328,7 @@ __device__ __forceinline__ uint32_t point_of_cloud(const FrameArgs &a, int64_t i
     return point_word(a, x, y, z, bit);
 }
 
-// Point i of the cloud.  Warp-synchronous like voxelize_depth_thread.
+// Point i of the cloud.  Warp-synchronous: every lane of the warp calls it.
 __device__ __forceinline__ void voxelize_points_thread(const FrameArgs &a, int64_t i) {
     uint32_t bit = 0;
     const uint32_t key = point_of_cloud(a, i, bit);

@@ -318,3 +318,33 @@ def test_batch_of_both_forms_at_odd_sizes(vg, copies):
         batch.close()
         for g in grids:
             g.close()
+
+
+def test_batch_of_images_of_few_rows_and_columns(vg):
+    # K1 takes such images' pixels as they lie in memory, next to tiled ones
+    from oracle import OracleGrid, OracleParams
+    rng = np.random.default_rng(9)
+    n, vs = (90, 70, 40), 0.1
+    shapes = [(3000, 1), (1, 3000), (1023, 7), (64, 48), (5, 211), (1, 1)]
+    grids = [vg.Grid(n, vs, 80, 60, 4.0, 1) for _ in shapes]
+    oracles = [OracleGrid(OracleParams(n, vs, 80, 60, 4.0, 1), (0.0, 0.0, 0.0)) for _ in shapes]
+    batch = vg.Batch(len(shapes))
+    try:
+        for step in range(2):
+            frames = []
+            for k, (w, h) in enumerate(shapes):
+                d = rng.uniform(0.3, 4.5, (h, w)).astype(np.float32)
+                if k % 2:
+                    d = np.rint(d * 1000).astype(np.uint16)
+                frames.append((grids[k], torch.from_numpy(d).cuda(), body_pose([0.0, 0.0, 0.0], step + k), None,
+                               1e-3 if k % 2 else 1.0))
+                oracles[k].integrate_depth(frames[-1][2], d, frames[-1][4])
+            batch.step(frames)
+        assert batch.status() == vg.VG_OK
+        for g, o in zip(grids, oracles):
+            got, origin = _read(g)
+            assert np.array_equal(got.reshape(o.loc.shape), o.loc)
+    finally:
+        batch.close()
+        for g in grids:
+            g.close()

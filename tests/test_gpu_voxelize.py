@@ -118,3 +118,66 @@ def test_images_around_tiles(vg, w, h, dtype):
             torch.cuda.synchronize()
             assert_same(out.cpu().numpy().reshape(g.shape), o.loc, "%dx%d, offset %d, flat %s" % (w, h, off, flat))
         g.close()
+
+
+# rows that begin on every pixel of a whole four, whose fours reach into the
+# rows before and after, and images that end inside one
+@pytest.mark.parametrize("w,h", [(3, 3), (5, 2), (29, 35), (30, 33), (33, 34), (34, 5), (35, 7), (127, 40)])
+@pytest.mark.parametrize("dtype", [np.float32, np.uint16])
+def test_images_of_odd_widths(vg, w, h, dtype):
+    n, vs = (96, 120, 120), 0.1
+    rng = np.random.default_rng(w * 1000 + h)
+    scale = 1e-3 if dtype == np.uint16 else 1.0
+    for off in (0, 1):
+        g = vg.Grid(n, vs, 80.0, 70.0, 4.0, 0, (0.0, 0.0, 0.0), flags=vg.VG_FLAG_STATS)
+        o = OracleGrid(OracleParams(n, vs, 80.0, 70.0, 4.0, 0), (0.0, 0.0, 0.0))
+        out = torch.empty(g.nvox, dtype=torch.uint8, device="cuda")
+        for k in range(2):
+            d = rng.uniform(0.4, 5.0, (h, w))
+            d[rng.random((h, w)) < 0.05] = 0
+            d = np.rint(d * 1000).astype(dtype) if dtype == np.uint16 else d.astype(dtype)
+            # valid depths before and after the image, which must set nothing
+            buf = torch.from_numpy(np.full(w * h + 9, 1000 if dtype == np.uint16 else 1.0, dtype)).cuda()
+            at = 4 + off
+            buf[at:at + w * h] = torch.from_numpy(d.reshape(-1)).cuda()
+            T = body_pose([0.0, 0.0, 0.0], rng.uniform(-3, 3), 0.2, 0.1)
+            g.integrate_depth(buf[at:at + w * h].view(h, w), T, scale)
+            o.integrate_depth(T, d, scale)
+            g.read(out)
+            torch.cuda.synchronize()
+            assert_same(out.cpu().numpy().reshape(g.shape), o.loc, "%dx%d, offset %d" % (w, h, off))
+        assert 0 < g.stats()["points_in_grid"] <= 2 * w * h
+        g.close()
+
+
+# images of a few rows or columns, whose pixels K1 takes as they lie in memory,
+# and one row or column more; page-locked images whose rows begin inside a
+# unit of the host link; addresses and lengths that are no whole fours
+@pytest.mark.parametrize("w,h", [(2000, 1), (1, 2000), (1025, 7), (7, 1025), (403, 8), (8, 403), (3, 3), (1024, 1), (65, 33)])
+@pytest.mark.parametrize("dtype", [np.float32, np.uint16])
+@pytest.mark.parametrize("host", [False, True])
+def test_images_taken_as_they_lie(vg, w, h, dtype, host):
+    n, vs = (96, 120, 120), 0.1
+    rng = np.random.default_rng(w * 1000 + h)
+    scale = 1e-3 if dtype == np.uint16 else 1.0
+    for off in (0, 1):
+        g = vg.Grid(n, vs, 80.0, 70.0, 4.0, 0, (0.0, 0.0, 0.0), flags=vg.VG_FLAG_STATS)
+        o = OracleGrid(OracleParams(n, vs, 80.0, 70.0, 4.0, 0), (0.0, 0.0, 0.0))
+        out = torch.empty(g.nvox, dtype=torch.uint8, device="cuda")
+        for k in range(2):
+            d = rng.uniform(0.4, 5.0, (h, w))
+            d[rng.random((h, w)) < 0.05] = 0
+            d = np.rint(d * 1000).astype(dtype) if dtype == np.uint16 else d.astype(dtype)
+            # valid depths before and after the image, which must set nothing
+            buf = torch.from_numpy(np.full(w * h + 9, 1000 if dtype == np.uint16 else 1.0, dtype))
+            buf = buf.pin_memory() if host else buf.cuda()
+            at = 4 + off
+            buf[at:at + w * h] = torch.from_numpy(d.reshape(-1))
+            T = body_pose([0.0, 0.0, 0.0], rng.uniform(-3, 3), 0.2, 0.1)
+            g.integrate_depth(buf[at:at + w * h].view(h, w), T, scale)
+            o.integrate_depth(T, d, scale)
+            g.read(out)
+            torch.cuda.synchronize()
+            assert_same(out.cpu().numpy().reshape(g.shape), o.loc, "%dx%d, offset %d" % (w, h, off))
+        assert 0 < g.stats()["points_in_grid"] <= 2 * w * h
+        g.close()
