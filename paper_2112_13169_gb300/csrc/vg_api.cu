@@ -639,6 +639,7 @@ int vg_integrate_depth(vg_grid *G, const void *depth, int32_t mem, int32_t width
         if (rc != VG_OK) return rc;
     }
     FrameArgs a = depth_frame_args(G, T, dptr, width, height, dtype, depth_scale);
+    if (mem == VG_MEM_HOST && dptr != G->staging) vg::host::over_link(a);
     gather_form(G, a);
     cudaError_t e = launch(G, VG_K_VOXELIZE, s, [&] { return vg::launch_voxelize_depth(a, dtype, s, G->sched); });
     if (e == cudaSuccess) e = finish_frame(G, a, s);

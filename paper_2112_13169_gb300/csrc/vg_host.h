@@ -172,6 +172,11 @@ inline void set_depth_frame(FrameArgs &a, const vg_params *p, const void *depth,
     depth_box(a, p, tx, ty);
 }
 
+// The image is read over the host link, in units of 32 bytes: a tile's rows
+// that begin inside them read a fourth more, pixels as they lie do not (16-bit
+// frames of 641x479: K1 14.4 us in tiles, 13.0 so; 640x480 12.1 and 12.4).
+inline void over_link(FrameArgs &a) { a.linear = a.linear || a.W % 16 != 0; }
+
 // Narrows a frame's box to a pyramid from the camera, of depth d voxels and
 // half sides kx and ky there, with `spare` voxels more for rounding.  Poses
 // whose rotation block is no rotation keep their linear map, so the corners

@@ -54,8 +54,9 @@ cudaError_t setup_device(int dev) {
 // The address at which the kernels on device `dev` reach p: p itself for
 // device (or managed) memory of that device, the mapped device address for
 // page-locked host memory when host_ok, else NULL (memory of another device,
-// pageable host memory, or a pointer CUDA does not know).  Allocates nothing.
-const void *reachable(const void *p, int dev, bool host_ok) {
+// pageable host memory, or a pointer CUDA does not know).  *host says whether
+// it is host memory.  Allocates nothing.
+const void *reachable(const void *p, int dev, bool host_ok, bool *host = nullptr) {
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();   // not a CUDA-known pointer: clear the error
@@ -63,7 +64,10 @@ const void *reachable(const void *p, int dev, bool host_ok) {
     }
     if (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged)
         return at.device == dev ? p : nullptr;
-    if (at.type == cudaMemoryTypeHost && host_ok) return at.devicePointer;
+    if (at.type == cudaMemoryTypeHost && host_ok) {
+        if (host) *host = true;
+        return at.devicePointer;
+    }
     return nullptr;
 }
 
@@ -91,7 +95,8 @@ extern "C" VG_API int vg_integrate_depth_noalloc(const vg_params *params, const 
     // the kernels run on the current device: loc must be its memory, and
     // depth its memory or page-locked host memory it reads in place
     uint8_t *dloc = static_cast<uint8_t *>(const_cast<void *>(reachable(loc, dev, false)));
-    const void *ddepth = reachable(depth, dev, true);
+    bool linked = false;
+    const void *ddepth = reachable(depth, dev, true, &linked);
     if (!dloc || !ddepth) return VG_EINVAL;
     e = setup_device(dev);
     if (e != cudaSuccess) return vg::host::status_of(e);
@@ -100,6 +105,7 @@ extern "C" VG_API int vg_integrate_depth_noalloc(const vg_params *params, const 
 
     vg::FrameArgs a = vg::host::frame_args(params, g, T);
     vg::host::set_depth_frame(a, params, ddepth, width, height, dtype, depth_scale);
+    if (linked) vg::host::over_link(a);
     a.pl.occ_raw = scratch;
     a.pl.occ_inf = scratch + g.words;
     a.pl.fr = scratch + 2 * g.words;

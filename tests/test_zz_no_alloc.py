@@ -139,3 +139,10 @@ def test_noalloc_refuses_grids_beyond_its_scratch(vg):
                                       vg.VG_DEPTH_F32, 1.0, T.ctypes.data_as(C.c_void_p), None)
     assert rc == vg.VG_ESCRATCH, rc
     assert vg.strerror(rc) == "grid too large for the fixed scratch array"
+
+
+def test_noalloc_reads_page_locked_rows_of_any_width(vg):
+    # rows that begin inside a unit of the host link
+    from synth import make
+    w = make("robot", robot=712, frames=2, spec=(323, 241, 0.1, (80, 80, 40), 1))
+    _check_calls(vg, w, range(2), depth_of=lambda f: torch.from_numpy(f.depth).pin_memory())
