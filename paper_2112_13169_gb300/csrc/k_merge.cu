@@ -41,10 +41,11 @@ __global__ void __launch_bounds__(256) k_loc_occupancy(const PlaneGeom g, const 
     out[w] = bits;
 }
 
+template <bool NARROW>
 __global__ void __launch_bounds__(256) k_shift(const PlaneGeom g, const Ring ring, const uint8_t *src, uint8_t *dst) {
     pdl_trigger();
     pdl_wait();
-    units::shift_chunk<units::LoadPlain>(g, ring, src, dst, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    units::shift_chunk<units::LoadPlain, NARROW>(g, ring, src, dst, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 template <int WPU>
@@ -75,7 +76,8 @@ cudaError_t launch_shift(const PlaneGeom &g, const Ring &ring, const uint8_t *sr
     const int64_t threads = (g.nvox + 15) / 16;
     const unsigned blocks = (unsigned)((threads + 255) / 256);
     if (blocks == 0) return cudaSuccess;
-    return launch_pdl(k_shift, blocks, 256, 0, s, g, ring, src, dst);
+    if (g.nx <= units::kNarrowRow) return launch_pdl(k_shift<true>, blocks, 256, 0, s, g, ring, src, dst);
+    return launch_pdl(k_shift<false>, blocks, 256, 0, s, g, ring, src, dst);
 }
 
 }  // namespace vg

@@ -178,3 +178,10 @@ def test_gathered_clouds_all_round(vg, n, r, off):
         P.o.shift(to)
     P.check("%s after the last re-centre" % (n,))
     P.g.close()
+
+
+@pytest.mark.parametrize("n", [(1, 40, 3), (2, 3, 11), (3, 7, 7), (4, 9, 4), (5, 9, 4), (1, 1, 1), (2, 1, 37)])
+def test_reads_of_narrow_rows_through_the_ring(vg, n):
+    # rows read voxel by voxel (up to four), and one by runs; chunks that end
+    # in a row, in a slice and past the grid
+    test_reads_through_the_ring(vg, n)
