@@ -368,7 +368,8 @@ VG_API int vg_batch_tune(vg_batch *batch, int32_t knob, int32_t value);
  * the occupancy limit), lanes per ray (per grid, 8, 16, 32), inflate tile
  * slices (8, 4), merge words per unit (512, 256), phase-3 spread (2, 1, 0)
  * -- with the other knobs at the best values found so far (coordinate
- * descent), keeps the fastest setting in the batch and writes it to best[5]
+ * descent; lanes, merge words and spread only if some frame is not gathered,
+ * see VG_TUNE_RT_LANES), keeps the fastest setting in the batch and writes it to best[5]
  * = {ctas_per_sm, lanes, inflate_slices, merge_words, spread} (may be NULL).
  * Synchronises the device.  Errors: as vg_batch_step, VG_ETIMEOUT.
  */
@@ -502,8 +503,8 @@ enum {
  * bracketed by two CUDA events recorded on the launch's own stream (up to
  * 65536 launches are kept; later ones are counted but not timed).
  * vg_profile_read synchronises the device, writes the summed event time in
- * milliseconds and the number of timed launches per kernel, and (if reset)
- * forgets them.  launches_total (may be NULL) receives the number of kernel
+ * milliseconds and the number of timed launches per kernel (a gathered frame's
+ * VG_K_RAYTRACE, two launches, is timed as one), and (if reset) forgets them.  launches_total (may be NULL) receives the number of kernel
  * launches this grid has issued since creation, timed or not.
  * Errors: VG_EINVAL, VG_ENOMEM (event pool), VG_ECUDA.
  */
@@ -518,10 +519,13 @@ VG_API int vg_profile_read(vg_grid *grid, double ms[VG_NKERNELS], int64_t timed[
  *                    lanes, at least 8, whose share of the longest ray is
  *                    at most 1.5 times the per-lane buffer of runs of
  *                    visits).  Results do not depend on it.  Large frames
- *                    trace without walking (K3 finds each ray's first
- *                    occupied voxel, K4 looks its rays up per voxel) unless
- *                    VG_FLAG_STATS counts visits; this knob, K3's CTAs per
- *                    SM and K4's words then have no effect.
+ *                    are gathered: they trace without walking (K3 finds each
+ *                    ray's first occupied voxel, K4 looks its rays up per
+ *                    voxel), and this knob, K3's CTAs per SM and K4's words
+ *                    have no effect.  Grids with flags, poses that are no
+ *                    rotation, views of more than 105 degrees and sides,
+ *                    ranges or camera distances of more than 4096 voxels
+ *                    always walk.
  *  VG_TUNE_INFLATE_TILE
  *                    K2's tile of plane words: VG_TILE_AUTO (the default:
  *                    8 words x 8 rows x 8 slices, 4 slices when the grid has
@@ -563,7 +567,8 @@ VG_API int vg_tune(vg_grid *grid, int32_t knob, int32_t value);
  * schedule as it stands, it takes one knob at a time -- K2's tile (the four
  * shapes), K3's lanes per ray (8, 16, 32), K3's CTAs per SM (1..5), K4's
  * words per CTA (256, 512), K2's staging (tensor copies or threads) and
- * K2's launch (while K1 runs or after it) --
+ * K2's launch (while K1 runs or after it) -- but lanes, CTAs per SM and K4's
+ * words only for a frame that is not gathered (VG_TUNE_RT_LANES) --
  * and compares each candidate value with the best schedule so far: `reps`
  * (1 .. 1000) measurements of the given depth frame (arguments as for
  * vg_integrate_depth) under each, alternating and each in turn first,

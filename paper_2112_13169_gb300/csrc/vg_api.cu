@@ -581,10 +581,20 @@ int vg_autotune(vg_grid *G, const void *depth, int32_t mem, int32_t width, int32
     const int tma[2] = {1, 0};
     const int early[2] = {1, 0};
     vg::Sched bs = G->sched;
+    // passes 1 to 3 are K3's and K4's in their walked form: on a frame that is
+    // gathered they would compare a schedule with itself
+    vg::Pose32 T;
+    bool gathered = false;
+    if (pose_of(G, T_wc, T)) {
+        FrameArgs a = depth_frame_args(G, T, depth, width, height, dtype, depth_scale);
+        gather_form(G, a);
+        gathered = a.ga.on;
+    }
     int bl = G->lanes_per_ray ? G->lanes_per_ray : vg::auto_lanes_per_ray(G->vd, G->hw, G->hh);
     for (int pass = 0; pass < 6 && rc == VG_OK; ++pass) {
         const int n = pass == 0 ? 4 : (pass == 1 ? 3 : (pass == 2 ? 5 : 2));
         if ((pass == 0 || pass == 4) && G->p.vox_inf == 0) continue;   // no K2 to tune
+        if (pass >= 1 && pass <= 3 && gathered) continue;
         for (int i = 0; i < n && rc == VG_OK; ++i) {
             vg::Sched sc = bs;
             int lp = bl;
@@ -1112,6 +1122,9 @@ int vg_batch_autotune(vg_batch *B, const vg_frame *frames, int32_t n, int32_t re
     for (int k = 0; k < 5 && rc == VG_OK; ++k) {
         int pick[5];
         std::memcpy(pick, cur, sizeof(pick));
+        // lanes, merge words and the spread are for walked frames: a batch of
+        // gathered ones (no units of the walked phase 3) does not depend on them
+        if (k != 0 && k != 2 && reinterpret_cast<const vg::BatchCtl *>(B->host)->total[2] == 0) continue;
         for (size_t i = 0; i < cand[k].size() && rc == VG_OK; ++i) {
             int v[5];
             std::memcpy(v, cur, sizeof(v));

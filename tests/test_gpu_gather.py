@@ -185,3 +185,32 @@ def test_reads_of_narrow_rows_through_the_ring(vg, n):
     # rows read voxel by voxel (up to four), and one by runs; chunks that end
     # in a row, in a slice and past the grid
     test_reads_through_the_ring(vg, n)
+
+
+def test_autotune_of_a_gathered_frame_leaves_the_walk_alone(vg):
+    # lanes, K3's CTAs and K4's words do nothing on a gathered frame: their
+    # candidates are not timed, and none is picked on noise
+    w = make("seq", frames=1)
+    g, f, reps = w.grid, w.frames[0], 2
+    G = vg.Grid(g.n, g.vox_size, w.cam.fov_x, w.cam.fov_y, g.depth, g.vox_inf, f.robot_pos)
+    best = G.autotune(torch.from_numpy(f.depth).cuda(), f.T_wc, reps=reps)
+    assert (best["ctas_per_sm"], best["merge_words"]) == (0, 256) and best["lanes"] == 8
+    # four tiles, K2's staging and its launch, each against the best so far,
+    # reps and one frames of both
+    frames = (4 + 1 + 1) * 2 * (reps + 1)
+    launches = {k: v[2] for k, v in G.profile_read().items()}
+    assert launches["voxelize"] == frames and launches["raytrace"] == 2 * frames
+    G.close()
+
+
+def test_autotune_of_a_gathered_batch_leaves_the_walk_alone(vg):
+    w = make("seq", frames=1)
+    g, f = w.grid, w.frames[0]
+    grids = [vg.Grid(g.n, g.vox_size, w.cam.fov_x, w.cam.fov_y, g.depth, g.vox_inf, f.robot_pos) for _ in range(2)]
+    d = torch.from_numpy(f.depth).cuda()
+    batch = vg.Batch(2)
+    best = batch.autotune([(G, d, f.T_wc, None, 1.0) for G in grids], reps=2)
+    assert (best["lanes"], best["merge_words"], best["spread"]) == (0, 512, 1)
+    batch.close()
+    for G in grids:
+        G.close()
