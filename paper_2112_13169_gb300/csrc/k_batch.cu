@@ -11,7 +11,8 @@
 //   phase 3b K3 gathered           32 x 8 rays (their latest hits)
 //   phase 4  K4 gathered           192 plane words of the box; 256 of slabs
 //            K4 merge              512 plane words (256 if tuned)
-// with a grid-wide barrier between phases (3b only if a frame is gathered).
+// with a grid-wide barrier between phases (3b only if a frame is gathered; a
+// batch without gathered frames takes a kernel without their phases).
 // A batch whose frames that the gathered form can take (vg_gather.cuh) hold
 // enough voxels together (kBatchGatherVoxels) has them gathered: many frames
 // fill the device, so its fewer instructions count and the latency of its
@@ -163,6 +164,11 @@ __device__ __forceinline__ void stage_args(const FrameArgs &src, FrameArgs &dst)
     for (int k = threadIdx.x; k < (int)(sizeof(FrameArgs) / 4); k += kThreads) d[k] = __ldg(s + k);
 }
 
+// GATHER: some frame may be gathered.  Batches of walked frames alone, which
+// are small, take a kernel of their own: the gathered phases' code costs them
+// time although they run none of it (one 320x240 frame into 80 x 80 x 40 voxels
+// 43.9 us a step with it, 41.0 without; into 100 x 100 x 20 46.5 and 45.6).
+template <bool GATHER>
 __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restrict__ items, BatchCtl *ctl) {
     __shared__ uint32_t box_fr[kBoxWords], box_tr[kBoxWords], occ_box[kBoxWords];
     extern __shared__ __align__(16) uint32_t dyn[];
@@ -174,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
     // and per-ray code reads them there rather than field by field from the
     // table in global memory.
     __shared__ FrameArgs s_a;
-    __shared__ int32_t s_kind;   // phase 1: dtype * 2 + vec; phase 3: LPR * 2 + buffered
+    __shared__ int32_t s_kind;   // phase 1: dtype * 3 + pix_mode; phase 3: LPR * 2 + buffered
 
     // ---- phase 1: voxelize ------------------------------------------------
     {
@@ -193,7 +199,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
                 cur = i;
             }
             const int64_t local = u - __ldg(&items[i].off[0]), pix = __ldg(&items[i].pix_units);
-            if (local >= pix) {
+            if (GATHER && local >= pix) {
                 gather::table_thread(s_a, (local - pix) * kThreads + threadIdx.x);
                 ++u;
                 continue;
@@ -211,7 +217,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
             }
             u += run;
         }
-        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->next = 0u;   // phase 3 counts from 0
+        if (GATHER && blockIdx.x == 0 && threadIdx.x == 0) ctl->next = 0u;   // phase 3 counts from 0
     }
     if (!grid_sync(ctl, nb)) return;
 
@@ -269,7 +275,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
         __syncthreads();
         return (int64_t)s_next;
     };
-    {
+    if (GATHER) {
         float S[3];
         int32_t v0[3];
         uint32_t asked = 0;
@@ -293,8 +299,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
     // a contiguous run of units per CTA, so the camera box is staged again
     // only when the run crosses into another frame; the runs split the
     // units' total weight evenly (weights of 1: their number)
-    if (ctl->total[2])
-    {
+    if (!GATHER || ctl->total[2]) {
         const int64_t lo = weighted_unit(items, n, ctl->total[2], run_begin(ctl->wtotal3, blockIdx.x, nb));
         const int64_t hi = weighted_unit(items, n, ctl->total[2], run_begin(ctl->wtotal3, blockIdx.x + 1, nb));
         int cur = -1, i = find_item(items, n, 2, lo);
@@ -334,7 +339,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
     if (!grid_sync(ctl, nb)) return;
 
     // ---- phase 3b: the latest hits of the gathered frames' rays -----------
-    if (ctl->total[5]) {
+    if (GATHER && ctl->total[5]) {
         int i = 0;
         if (blockIdx.x == 0 && threadIdx.x == 0) ctl->next = 0u;   // and phase 4
         for (int64_t u = blockIdx.x; u < ctl->total[5]; u += nb) {
@@ -350,7 +355,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
     {
         float S[3];
         int32_t v0[3];
-        const bool handed = ctl->total[5] != 0;   // (a batch of scattered frames alone: in turn)
+        const bool handed = GATHER && ctl->total[5] != 0;   // (a batch of scattered frames alone: in turn)
         uint32_t asked = 0;
         int i = find_item(items, n, 3, blockIdx.x);
         for (int64_t u = blockIdx.x; u < ctl->total[3]; u = handed ? told(asked) : u + nb) {
@@ -358,7 +363,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const BatchItem *__restri
             const BatchItem &it = items[i];
             const int64_t local = u - __ldg(&it.off[3]);
             if (handed) asked = ask();
-            if (__ldg(&it.a.ga.on)) {
+            if (GATHER && __ldg(&it.a.ga.on)) {
                 stage(i);
                 const int32_t box = __ldg(&it.box_units);
                 if (local < box) {
@@ -386,10 +391,14 @@ int g_batch_sms[64];
 cudaError_t configure_batch(int dev) {
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     const size_t dyn = sizeof(uint32_t) * kDynWords;
-    cudaError_t e = cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_batch_sms[dev], cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_batch_blocks_per_sm[dev], k_batch, kThreads, dyn);
+    cudaError_t e = cudaDeviceGetAttribute(&g_batch_sms[dev], cudaDevAttrMultiProcessorCount, dev);
+    int per_sm[2] = {0, 0};
+    for (int k = 0; k < 2; ++k) {
+        auto kernel = k ? k_batch<true> : k_batch<false>;
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[k], kernel, kThreads, dyn);
+    }
+    g_batch_blocks_per_sm[dev] = per_sm[0] < per_sm[1] ? per_sm[0] : per_sm[1];
     return e;
 }
 
@@ -398,10 +407,10 @@ int batch_max_blocks(int dev) {
     return g_batch_sms[dev] * g_batch_blocks_per_sm[dev];
 }
 
-cudaError_t launch_batch(const BatchItem *items, BatchCtl *ctl, int blocks, cudaStream_t s) {
+cudaError_t launch_batch(const BatchItem *items, BatchCtl *ctl, int blocks, bool gather, cudaStream_t s) {
     void *args[] = {(void *)&items, (void *)&ctl};
-    return cudaLaunchCooperativeKernel((const void *)k_batch, dim3(blocks), dim3(kThreads), args,
-                                       sizeof(uint32_t) * kDynWords, s);
+    return cudaLaunchCooperativeKernel((const void *)(gather ? k_batch<true> : k_batch<false>), dim3(blocks), dim3(kThreads),
+                                       args, sizeof(uint32_t) * kDynWords, s);
 }
 
 }  // namespace vg

@@ -930,7 +930,7 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
     vg::BatchCtl *ctl = reinterpret_cast<vg::BatchCtl *>(B->host);
     vg::BatchItem *items = reinterpret_cast<vg::BatchItem *>(B->host + sizeof(vg::BatchCtl));
     int64_t total[6] = {0, 0, 0, 0, 0, 0};
-    double voxels = 0.0;   // of the frames that could be gathered
+    double most = 0.0;   // voxels of the frames that may be gathered
     for (int32_t i = 0; i < n; ++i) {
         const vg_frame &f = frames[i];
         vg_grid *G = f.grid;
@@ -939,8 +939,14 @@ int vg_batch_prepare(vg_batch *B, const vg_frame *frames, int32_t n) {
         vg::BatchItem &it = items[i];
         std::memset(&it, 0, sizeof(it));
         it.a = depth_frame_args(G, T, f.depth, f.width, f.height, f.dtype, f.depth_scale);
-        if (G->p.flags == 0) vg::host::gather_setup(it.a, G->loc_alt, (size_t)G->g.nvox + 16);
-        if (it.a.ga.on) voxels += vg::host::gather_voxels(it.a);
+        if (G->p.flags == 0) most += vg::host::gather_voxels(it.a);
+    }
+    double voxels = 0.0;   // of those that can be
+    for (int32_t i = 0; i < n && most >= vg::host::kBatchGatherVoxels; ++i) {
+        vg_grid *G = frames[i].grid;
+        FrameArgs &a = items[i].a;
+        if (G->p.flags == 0) vg::host::gather_setup(a, G->loc_alt, (size_t)G->g.nvox + 16);
+        if (a.ga.on) voxels += vg::host::gather_voxels(a);
     }
     const bool gather = voxels >= vg::host::kBatchGatherVoxels;
     for (int32_t i = 0; i < n; ++i) {
@@ -1053,12 +1059,15 @@ int vg_batch_enqueue(vg_batch *B, void *stream) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     e = cudaStreamIsCapturing(s, &cs);
     if (e != cudaSuccess) return status_of(e);
-    const unsigned rec = (cs == cudaStreamCaptureStatusActive) ? cudaEventRecordExternal : cudaEventRecordDefault;
+    const bool captured = cs == cudaStreamCaptureStatusActive;
+    const unsigned rec = captured ? cudaEventRecordExternal : cudaEventRecordDefault;
+    // a graph runs whatever later steps prepare, so it takes the kernel for both
+    const bool gather = captured || reinterpret_cast<const vg::BatchCtl *>(B->host)->total[5] != 0;
     e = cudaMemcpyAsync(B->dev, B->host, B->bytes, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaEventRecordWithFlags(B->copied, s, rec);
     if (e == cudaSuccess)
         e = vg::launch_batch(reinterpret_cast<const vg::BatchItem *>(B->dev + sizeof(vg::BatchCtl)),
-                             reinterpret_cast<vg::BatchCtl *>(B->dev), blocks, s);
+                             reinterpret_cast<vg::BatchCtl *>(B->dev), blocks, gather, s);
     if (e == cudaSuccess) e = cudaEventRecordWithFlags(B->done, s, rec);
     if (e != cudaSuccess) return status_of(e);
     B->enqueued = true;

@@ -252,6 +252,7 @@ cudaError_t launch_loc_occupancy(const PlaneGeom &g, const uint8_t *loc, const R
                                  cudaStream_t s);
 cudaError_t configure_batch(int dev);   // once per device, before the first launch_batch
 int batch_max_blocks(int dev);          // CTAs of k_batch resident at once on the device
-cudaError_t launch_batch(const BatchItem *items, BatchCtl *ctl, int blocks, cudaStream_t s);
+// gather: whether any item may be gathered
+cudaError_t launch_batch(const BatchItem *items, BatchCtl *ctl, int blocks, bool gather, cudaStream_t s);
 
 }  // namespace vg

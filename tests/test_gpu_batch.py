@@ -348,3 +348,41 @@ def test_batch_of_images_of_few_rows_and_columns(vg):
         batch.close()
         for g in grids:
             g.close()
+
+
+def test_a_captured_step_runs_whatever_is_prepared_later(vg):
+    # a graph captured over a batch of small frames (walked) is replayed over
+    # one of large frames (gathered), and the other way round
+    from oracle import OracleGrid, OracleParams
+    rng = np.random.default_rng(15)
+    P = {False: ((60, 50, 30), 0.1, 80, 60, 3.0, 1), True: ((200, 200, 100), 0.05, 87, 58, 5.0, 2)}
+
+    def frame(large, yaw):
+        d = (rng.uniform(0.3, 1.1, (48, 64)) * P[large][4]).astype(np.float32)
+        return torch.from_numpy(d).cuda(), body_pose([0.0, 0.0, 0.0], yaw), d
+
+    for first in (False, True):
+        grids = {k: vg.Grid(*P[k][:5], P[k][5]) for k in P}
+        oracles = {k: OracleGrid(OracleParams(*P[k]), (0.0, 0.0, 0.0)) for k in P}
+        batch = vg.Batch(1)
+        stream = torch.cuda.Stream()
+        seq = [first, not first, first, not first]
+        frames = [frame(k, 0.7 * i) for i, k in enumerate(seq)]
+        graph = torch.cuda.CUDAGraph()
+        batch.prepare([(grids[first], frames[0][0], frames[0][1], None, 1.0)])
+        with torch.cuda.graph(graph, stream=stream):
+            batch.enqueue()
+        for i, k in enumerate(seq):
+            if i:
+                torch.cuda.synchronize()
+                batch.prepare([(grids[k], frames[i][0], frames[i][1], None, 1.0)])
+            graph.replay()
+            torch.cuda.synchronize()
+            assert batch.status() == vg.VG_OK
+            oracles[k].integrate_depth(frames[i][1], frames[i][2])
+        for k in P:
+            got, _ = _read(grids[k])
+            assert np.array_equal(got.reshape(oracles[k].loc.shape), oracles[k].loc), (first, k)
+        batch.close()
+        for g in grids.values():
+            g.close()
