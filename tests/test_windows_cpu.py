@@ -142,3 +142,18 @@ def test_faces_beside_and_behind_the_camera_have_no_rays(win, frame):
     for k in range(3):
         w = faces(win, i, np.full(len(i), k))
         assert ((w[:, 0] > w[:, 1]) | (w[:, 2] > w[:, 3])).all()
+
+
+def test_the_smallest_mixed_batch_is_gathered(win):
+    # the frames of test_batch_of_both_forms_at_odd_sizes, one of each: the
+    # batch has to take the gathered form, and one of its frames the walked
+    from test_gpu_batch import BOTH
+    win.w_gather_voxels.restype = win.w_batch_rule.restype = C.c_double
+    voxels = []
+    for k, (n, vs, fov, r, (w, h)) in enumerate(BOTH):
+        pos = np.array((0.0, -0.2 * k, 0.1))
+        origin = (np.floor(pos / np.float64(np.float32(vs))) - np.array(n) // 2).astype(np.int32)
+        T = np.ascontiguousarray(body_pose(pos + 0.03, k), np.float64)
+        voxels.append(win.w_gather_voxels(ptr(np.array(n, np.int32)), C.c_float(vs), C.c_float(fov), C.c_float(fov - 20),
+                                          C.c_float(np.float32(0.45 * max(n) * vs)), r, ptr(T), ptr(origin), w, h))
+    assert min(voxels) == 0.0 and sum(voxels) >= win.w_batch_rule()

@@ -55,6 +55,20 @@ void w_voxels(int64_t m, const int32_t *i, int32_t *out) {
     }
 }
 
+// The voxels by which a depth frame of the same grid and pose counts for the
+// gathered form (0: it is walked), and the sum from which a batch is gathered.
+double w_gather_voxels(const int32_t n[3], float vs, float fx, float fy, float depth, int32_t r, const double T_wc[16],
+                       const int32_t origin[3], int32_t w, int32_t h) {
+    vg_params p = {{n[0], n[1], n[2]}, vs, fx, fy, depth, r, 0};
+    Pose32 T;
+    if (!host::shape_ok(&p) || !host::pose_vc(T_wc, origin, vs, T)) return -1.0;
+    FrameArgs a = host::frame_args(&p, host::geom_of(&p), T);
+    host::set_depth_frame(a, &p, reinterpret_cast<const void *>(256), w, h, VG_DEPTH_F32, 1.0f);
+    host::gather_setup(a, reinterpret_cast<uint8_t *>(256), (size_t)a.g.nvox + 16);
+    return a.ga.on ? host::gather_voxels(a) : 0.0;
+}
+double w_batch_rule() { return host::kBatchGatherVoxels; }
+
 uint32_t w_round_entries(int32_t rays) { return gather::round_entries(rays); }
 int32_t w_max_rays() { return kMaxRays; }
 void w_rows(int64_t m, const uint32_t *q, const uint32_t *na, int32_t rays, uint32_t *out) {
