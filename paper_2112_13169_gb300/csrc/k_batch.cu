@@ -23,8 +23,11 @@
 // CTA finds the frame of its first unit of a phase by binary search, steps
 // forward through the frames as its units advance (see run_begin), and runs
 // the same device code as the one-step kernels (vg_units.cuh, vg_rt.cuh).
-// The merge's reads of data an earlier phase wrote skip the L1 (LoadL2);
-// for the inflation's and the rays' loads see there (and group_lpr).
+// Reads of data an earlier phase wrote: the walked frames' merge skips the L1
+// (LoadL2).  The inflation's and the rays' loads go through it, and the
+// gathered phases' (hits, 1/D with the latest hits, tiles, near words), which
+// loaded some of those lines before they were written: that they see the new
+// state rests on the barrier's fences (vg_sync.cuh).
 //
 // With 32 warps to an SM the phases are bound by latency more than by issue
 // (313 M warp instructions in 529 us, 54 % of the issue slots, for 64

@@ -10,7 +10,8 @@ namespace {
 // K1 lets the frame's later kernels launch only once the work before the
 // frame has completed: with `early` right after its own wait, so that K2's
 // launch overlaps K1; without, when K1 completes, which leaves K1's SM
-// slots to K3's CTAs, whose walk runs before they wait for K2.
+// slots to K3's CTAs, whose walk runs before they wait for K2 (a gathered
+// frame's K3 does nothing before its wait).
 //
 // The first `ntab` CTAs write the gathered form's ray table instead.
 template <int DT, int MODE>

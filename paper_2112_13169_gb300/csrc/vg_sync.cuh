@@ -1,5 +1,9 @@
-// vg_sync.cuh -- the grid-wide barrier of the persistent, cooperative
-// launches (k_batch.cu, k_frame.cu).
+// vg_sync.cuh -- the grid-wide barrier of the persistent, cooperative launch
+// (k_batch.cu).
+//
+// Between a CTA's arrival and its leaving stand device-scope fences, which
+// also drop the SM's L1: what any CTA wrote before the barrier, every CTA's
+// ordinary loads see after it, also of lines the SM held before.
 //
 // The CTAs arrive on a counter in global memory; the last of the
 // gridDim.x + bar_extra arrivals resets the counter and opens the next

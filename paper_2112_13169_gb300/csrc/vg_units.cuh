@@ -3,7 +3,9 @@
 // fused persistent launch (k_batch.cu).
 //
 // Loads of data that an earlier launch or phase wrote go through a load
-// policy: LoadPlain (ordinary loads) or LoadL2 (loads that skip the SM's L1).
+// policy: LoadPlain (ordinary loads) or LoadL2 (loads that skip the SM's L1;
+// ordinary ones see what was written before a grid barrier as well, by its
+// fences).
 // None take the read-only path: it is for data that nothing writes while the
 // kernel lives, and the one-step kernels are dependent launches, alive while
 // the kernel before them still writes.
