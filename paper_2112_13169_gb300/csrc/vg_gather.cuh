@@ -22,7 +22,7 @@
 //
 // Measured on a 640x480 frame into 200 x 200 x 100 voxels (21,201 rays of
 // 100; ncu): K3 10 + 5 us and K4 16 us here, K3 40 and K4 7.4 us scattered; on
-// 848x480 into 500 x 500 x 150 (132,525 rays of 250): 31 + 6 and 64 us against
+// 848x480 into 500 x 500 x 150 (132,525 rays of 250): 27 + 6 and 65 us against
 // 269 and 22.  Both are bound by instruction issue and the latency of their
 // phases, not by DRAM (1.1 MB a launch).
 //
